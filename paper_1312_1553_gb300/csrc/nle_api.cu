@@ -191,6 +191,10 @@ struct nle_ctx {
   DBuf d_perm, d_iperm;
   DBuf A_sptr, A_col, A_val, A64_val, d_diag;
   DBuf L_off, L_w, L_col, L_val, L_round, U_off, U_w, U_col, U_val, U_round;
+  // step form of the level schedule (first steps, heads, rows, operands,
+  // values, halo pointers and positions; L then U)
+  DBuf step_buf[2][7];
+  int steps = 0, halo_n = 0, step_n = 0, step_warps = 0;
   DBuf L_wp, L_task, U_wp, U_task;  // chain schedule: per-warp task lists
   int chain = 0;                     // schedule of the triangular solves in use (1 = chain)
   int trows = TRSV_ROWS;             // level schedule: rows a warp takes at a time (4 or 2)
@@ -294,6 +298,19 @@ static Dev<T> make_dev(nle_t h) {
   D.Uwp = h->U_wp.as<int32_t>();
   D.Ltask = h->L_task.as<int2>();
   D.Utask = h->U_task.as<int2>();
+  D.steps = h->steps;
+  D.step_n = h->step_n;
+  D.step_warps = h->step_warps;
+  for (int d = 0; d < 2; d++) {
+    TriSteps<T> &t = d ? D.SU : D.SL;
+    t.step0 = h->step_buf[d][0].as<int32_t>();
+    t.head = h->step_buf[d][1].as<StepHead>();
+    t.row = h->step_buf[d][2].as<int32_t>();
+    t.opnd = h->step_buf[d][3].as<int32_t>();
+    t.val = h->step_buf[d][4].as<T>();
+    t.hptr = h->step_buf[d][5].as<int32_t>();
+    t.hpos = h->step_buf[d][6].as<int32_t>();
+  }
   const int64_t np = h->npad, ext = h->npad + 32 * h->vw;
   T *v = h->vecs.as<T>();
   D.p = v + 0 * np;
@@ -341,13 +358,44 @@ static Opts make_opts(nle_t h, double tol, int max_newton, int max_pcg) {
   return O;
 }
 
+// Dynamic shared memory of the persistent kernels: two slab-sized buffers of
+// the triangular solves or, in the step form, the window of a solve slab (own
+// results, zero, halo).
+static size_t slab_smem(nle_t h) {
+  return (size_t)(h->steps ? h->bsize * h->steps + 1 + h->halo_n : 2 * h->bsize) * (mixed(h) ? 4 : 8);
+}
+constexpr size_t SLAB_SMEM_MAX = 192 * 1024;  // beside the kernels' static arrays (30 KB of 227)
+
+// Slabs per solve slab: a value takes about 1 us from one solve slab to the
+// next, so fewer of them are better as long as a level still is one step of
+// a warp.  Measured per application (mixed) with 1 / 2 / 4 slabs: 2D 600 x 700
+// (4.5 rows per level of a slab) 0.97 / 0.82 / 0.73 ms, 7-point 64^3 (9 rows)
+// 0.58 / 0.50 / 0.53, 7-point 100^3 (22 rows) 0.89 / 0.93 / 1.21, 27-point 48^3
+// (wide rows, two lanes each) 0.55 / 0.57 / 0.63.  FP64 is bound by its
+// arithmetic, 600 x 700: 3.10 / 3.19 / 3.28.
+static int solve_slabs(nle_t h, const Permuted &P) {
+  if (!mixed(h) || h->trows == 2) return 1;
+  int m = 1;
+  for (; m < 4; m *= 2) {
+    const int64_t rows = h->bsize * m * 2;
+    std::vector<int64_t> seen(h->F.nlevL, -1);
+    int64_t levels = 0;
+    for (int64_t i = 0; i < P.n; i++)
+      if (seen[P.lev[i]] != i / rows) {
+        seen[P.lev[i]] = i / rows;
+        levels++;
+      }
+    if (P.n > 20 * levels) break;
+  }
+  return m;
+}
+
 // Cooperative launch of kernel `id` (persistent, gridDim = h->grid).
 template <typename T>
 static nle_status launch(nle_t h, int id, void **args) {
   void *fn = kernel_ptr<T>(id, h->rpc, h->chain);
   if (!fn) return fail(h, NLE_ERR_ARG, "no kernel instance for this size");
-  // dynamic shared memory: two slab-sized buffers of the triangular solves
-  const size_t dyn = 2 * (size_t)h->bsize * (mixed(h) ? 4 : 8);
+  const size_t dyn = slab_smem(h);
   NLE_CUDA(h, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
   int nb = 0;
   NLE_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, TPB, dyn));
@@ -419,7 +467,29 @@ template <typename TV>
 static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, int chain) {
   const int H = 32 * h->vw;
   SellSet<TV> S;
-  build_sell<TV>(P, H, h->bsize, level_rounds, h->trows, S);
+  // step form of the level schedule where the window of a solve slab (own
+  // results and halo) fits in shared memory.  FP64 factors with wide rows (2
+  // rows per warp step) keep the polled form: eight lanes per row, ten FP64
+  // instructions of 64 cycles on the chain, measured 1.57 against 1.60 ms per
+  // application (27-point 48^3) but 1.85 against 1.78 ms per inner iteration.
+  StepsHost<TV> G[2];
+  const int lpr = sizeof(TV) == 8 ? 4 : h->trows == 2 ? 2 : 1;  // lanes per row of trsv_steps
+  h->steps = h->halo_n = 0;
+  if (!chain && !(sizeof(TV) == 8 && h->trows == 2)) {
+    h->step_warps = std::max(1, std::min(STEP_WARPS, h->opt.trsv_warps));
+    for (int m = solve_slabs(h, P); m >= 1; m /= 2) {
+      h->halo_n = h->step_n = 0;
+      for (int d = 0; d < 2; d++) {
+        plan_steps<TV>(P, h->bsize * m, d == 0, lpr, h->step_warps, G[d]);
+        h->halo_n = (int)std::max<int64_t>(h->halo_n, G[d].halo_max);
+        h->step_n = std::max(h->step_n, G[d].n_max);
+      }
+      h->steps = m;
+      if (slab_smem(h) <= SLAB_SMEM_MAX) break;
+      h->steps = 0;
+    }
+  }
+  build_sell<TV>(P, H, h->bsize, level_rounds, h->trows, S, !h->steps);
   NLE_CUDA(h, upload(h->A_sptr, S.A.sptr, h->stream));
   NLE_CUDA(h, upload(h->A_col, S.A.col, h->stream));
   NLE_CUDA(h, upload(h->A_val, S.A.val, h->stream));
@@ -439,6 +509,20 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
     NLE_CUDA(h, upload(h->U_task, CU.task, h->stream));
     S.L.round.assign(1, 0);
     S.U.round.assign(1, 0);
+  }
+  if (h->steps) {
+    for (int d = 0; d < 2; d++) {
+      StepsHost<TV> &g = G[d];
+      build_steps<TV>(P, h->bsize * h->steps, d == 0, lpr, g);
+      NLE_CUDA(h, upload(h->step_buf[d][0], g.step0, h->stream));
+      NLE_CUDA(h, upload(h->step_buf[d][1], g.head, h->stream));
+      NLE_CUDA(h, upload(h->step_buf[d][2], g.row, h->stream));
+      NLE_CUDA(h, upload(h->step_buf[d][3], g.opnd, h->stream));
+      NLE_CUDA(h, upload(h->step_buf[d][4], g.val, h->stream));
+      NLE_CUDA(h, upload(h->step_buf[d][5], g.hptr, h->stream));
+      NLE_CUDA(h, upload(h->step_buf[d][6], g.hpos, h->stream));
+    }
+    return NLE_OK;
   }
   NLE_CUDA(h, upload(h->L_off, S.L.off, h->stream));
   NLE_CUDA(h, upload(h->L_w, S.L.width, h->stream));
@@ -1209,7 +1293,7 @@ static nle_status batch_impl(int count, nle_t *hs, int p, double tol, int max_ne
     NLE_CUDA(h0, cudaMemsetAsync(h->state.p, 0, sizeof(State), h->stream));
     NLE_CUDA(h0, cudaStreamSynchronize(h->stream));
     while ((int64_t)rpc * h->grid * TPB < h->nchunks) rpc *= 2;
-    dyn = std::max(dyn, 2 * (size_t)h->bsize * sizeof(T));
+    dyn = std::max(dyn, slab_smem(h));
     order[b] = b;
   }
   if (rpc > 8) return fail(h0, NLE_ERR_ARG, "a problem is too large for its CTA group");

@@ -182,7 +182,10 @@ struct Shared {
   int ok;                      // error word broadcast after each barrier
   long long tlast;             // phase timer (CTA 0, thread 0)
   long long tacc[8];
+  int fin[64];                 // step solves: 1 + the last finished step of every step number modulo 64
+  alignas(16) int arrived[4];  // step solves: first missing halo value of each copying warp
 };
+static_assert(COPY_WARPS == 4, "arrived[] is read as one int4");
 
 struct Ctl {
   unsigned epoch;  // barriers passed by this CTA (thread 0 only)

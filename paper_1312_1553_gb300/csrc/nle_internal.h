@@ -48,6 +48,33 @@ struct Sell {
   const T *val = nullptr;
 };
 
+// Steps of a strictly triangular factor (see trsv_steps; cut by plan_steps).
+struct StepHead {
+  int32_t off;     // first quad of the step
+  uint32_t sync;   // threads of the barrier the step begins with (bits 0-9, 0: none); barriers it arrives at when it
+                   // ends: the first one's warp (10-13), their number (14-17) and threads (18-27)
+  uint32_t shape;  // lanes (bits 0-5), entries of a lane (6-15), flags (16-18)
+  int32_t need;    // halo values that must have arrived
+  int32_t first;   // first step of this level, in the solve slab
+  int32_t prev;    // first step of the level before it, in the solve slab
+  int32_t pad[2];
+};
+constexpr uint32_t STEP_REPORT = 1;  // more steps in the level than one barrier joins: reports its end
+constexpr uint32_t STEP_EARLY = 2;   // releases the next step, of the same level
+constexpr uint32_t STEP_WAIT = 4;    // a level with reports before: waits for them
+constexpr int COPY_WARPS = 4;        // warps of a CTA that copy the halo
+constexpr int STEP_WARPS = NWARP - COPY_WARPS;  // most solving warps (one named barrier each)
+template <typename T>
+struct TriSteps {
+  const int32_t *step0;  // per solve slab: first step
+  const StepHead *head;
+  const int32_t *row;    // 32 / lpr per step: the step's rows, in the solve slab
+  const int32_t *opnd;   // operands: bytes from the start of the window
+  const T *val;
+  const int32_t *hptr;  // per solve slab: first halo value
+  const int32_t *hpos;  // positions of the halo values
+};
+
 // Persistent solver state in device memory.  Written by CTA 0 only, at
 // points separated from every reader by a grid barrier or a kernel boundary.
 struct State {
@@ -123,6 +150,11 @@ struct Dev {
   const T *rdiag = nullptr;  // reciprocal diagonal of L (1 on padding rows)
   const uint16_t *Lround = nullptr, *Uround = nullptr;
   int trows = TRSV_ROWS;  // level schedule: rows a warp takes at a time (4, or 2 for wide rows)
+  // step form of the level schedule (steps > 0): the triangular factors as
+  // steps for solve slabs of `steps` slabs each, at most step_n entries per
+  // lane, for step_warps solving warps; the ELL arrays above are then unused
+  int steps = 0, step_n = 0, step_warps = 0;
+  TriSteps<T> SL{}, SU{};
   // chain schedule (chain = 1): the device order is the factored matrix's
   // own row order, and each slab's rows are solved as per-warp task lists
   // (Lwp/Uwp: NWARP + 1 offsets per slab into Ltask/Utask, a task = {first

@@ -230,8 +230,454 @@ extern __shared__ __align__(16) unsigned char nle_dyn_smem[];  // two slabs of t
 #endif
 constexpr bool kChainTU = NLE_CHAIN_TU != 0;
 
+// ---------------------------------------------------------------------------
+// Step form of the level schedule, one solve slab of rows per CTA.
+//
+// Solving a slab is a chain of levels, a few rows to a few dozen each, so what
+// counts is the time from one level to the next, and nothing on that path may
+// wait on global memory.
+//  * The first warps solve, taking the slab's steps (plan_steps) in turn: up to
+//    32 rows of one level.  All operands come from the slab's shared-memory
+//    window, results go to the window and, for the other slabs, to global
+//    memory.  A warp has the coefficients and operand addresses of its step
+//    in registers (loaded while the others work) when the level before ends:
+//    the warps of that level's steps arrive at a named barrier on which the
+//    warp of the next level's first step waits, and that one releases the
+//    next step of its level, and so on.  (A level with more steps than warps
+//    joins through reports in sh.fin instead.)
+//  * COPY_WARPS warps copy the halo, the values the slab needs from other
+//    slabs, from global memory into the window as they are published (a
+//    value is its own ready flag), and publish the first value of their share
+//    still missing.  A step states how many halo values it and the steps
+//    before it need, and its warp waits for them before it takes over.
+// A value takes about 1 us from one slab to the next, as long as some eight
+// levels, so a solve slab is several slabs (and fewer CTAs solve) where the
+// levels are narrow.
+//
+// Every wait ends: the steps of a slab follow the level order, and the halo
+// values listed up to a step belong to rows of lower levels than that step's,
+// so the unfinished row of lowest level always gets its inputs; all CTAs are
+// resident (cooperative launch).  The waits on flags are also bounded in
+// time; past the bound the warps go on without waiting, so that every warp
+// takes all its steps and the barriers between the warps always complete.
+// Barriers and votes need whole warps: what decides a wait is the same value
+// in all lanes, and the warp converges before them.
+//
+// Sums are formed as the 8-lane (16-lane) reduction of trsv_block forms them:
+// entry k of a row in partial sum k mod 8 (16), each partial sum in ascending
+// k, the partial sums added pairwise in the order of its butterfly, so both
+// forms give the same bits.  With LPR lanes per row, lane g holds the partial
+// sums p with p mod LPR = g: the first additions are in the lane, the others
+// between lanes.  FP32: one (two) lanes, since a shuffle costs as much as six
+// additions.  FP64: four, since an FP64 instruction occupies its quarter of
+// the SM for 64 cycles whatever the number of lanes (measured: 64 cycles for
+// one warp, 256 for four instructions, dependent or not).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// shared-memory accesses by 32-bit address, kept in program order
+__device__ __forceinline__ void lds(unsigned a, float &v) {
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds(unsigned a, double &v) {
+  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ int4 lds4(unsigned a) {
+  int4 v;
+  asm volatile("ld.volatile.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts(unsigned a, float v) {
+  asm volatile("st.volatile.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, double v) {
+  asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, int v) {
+  asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// Bound of a wait, asked every so many polls: true once spin_ns passed since
+// the first question or when another warp recorded an error.
+__device__ __forceinline__ bool wait_over(State *st, long long &t0, long long spin_ns, int where) {
+  const long long now = gtimer();
+  if (t0 == 0) t0 = now;
+  if (now - t0 > spin_ns) record_error(st, 8 /*NLE_ERR_TIMEOUT*/, where);
+  return ld_relaxed_int(&st->err) != 0;
+}
+
+// Copying warp m: its chunks of 32 halo values are m, m + COPY_WARPS, ...  One
+// chunk is in flight per warp: a pass over more of them costs every value
+// the whole pass, and the values arrive in nearly the order of the list.
 template <typename T>
-__device__ __forceinline__ void trsv_forward(const Dev<T> &D, Shared &sh, const Ctl &ctl, int k) {
+__device__ __forceinline__ void copy_halo(const int32_t *hpos, int nh, int m, const T *x, unsigned dst, Shared &sh,
+                                          long long spin_ns, State *st) {
+  const int lane = threadIdx.x & 31;
+  const unsigned flag = smem_addr(&sh.arrived[m]);
+  auto position = [&](int i) { return i < nh ? __ldg(hpos + i) : -1; };
+  int pos = position(32 * m + lane), ahead = position(32 * (m + COPY_WARPS) + lane);
+  for (int first = 32 * m; first < nh; first += 32 * COPY_WARPS) {
+    const unsigned to = dst + (unsigned)((first + lane) * (int)sizeof(T));
+    bool want = pos >= 0;
+    long long t0 = 0;
+    for (int it = 1;; it++) {
+      T v = T(0);
+      if (want) v = ld_relaxed(x + pos);
+      const bool got = want && !is_sent(v);
+      if (got) sts(to, v);
+      want = want && !got;
+      const unsigned left = __ballot_sync(0xffffffffu, want);
+      if (__any_sync(0xffffffffu, got)) {
+        __threadfence_block();
+        __syncwarp();
+        // all of this warp's values before the published one have arrived
+        if (lane == 0) sts(flag, left ? first + __ffs(left) - 1 : min(nh, first + 32 * COPY_WARPS));
+      }
+      if (!left) break;
+      if ((it & 4095) == 0 && __any_sync(0xffffffffu, wait_over(st, t0, spin_ns, 103))) {
+        if (want) sts(to, T(0));
+        break;
+      }
+    }
+    pos = ahead;
+    ahead = position(first + 64 * COPY_WARPS + lane);
+  }
+  __threadfence_block();
+  __syncwarp();
+  if (lane == 0) sts(flag, nh);
+}
+
+// Waits until the slab's steps from `from` up to `last` have reported their
+// end.  Step x of a warp is done when its next one (x + number of warps) has
+// begun, so the 32 steps up to `last` are enough.  Bounded.
+__device__ __forceinline__ void await_steps(const Shared &sh, int from, int last, long long spin_ns, State *st) {
+  const int x = last - (int)(threadIdx.x & 31);
+  const volatile int *f = &sh.fin[x & 63];
+  long long t0 = 0;
+  for (int it = 1;; it++) {
+    if (__all_sync(0xffffffffu, x < from || *f > x)) break;
+    if ((it & 4095) == 0 && __any_sync(0xffffffffu, wait_over(st, t0, spin_ns, 105))) break;
+  }
+  __threadfence_block();
+}
+
+// Waits until `need` halo values have arrived; returns how many have (the
+// same value in all lanes).  Bounded.
+__device__ __forceinline__ int await_halo(const Shared &sh, int need, long long spin_ns, State *st) {
+  const unsigned arrived = smem_addr(&sh.arrived[0]);
+  long long t0 = 0;
+  for (int it = 1;; it++) {
+    const int4 f = lds4(arrived);
+    const int here = (int)__reduce_min_sync(0xffffffffu, (unsigned)min(min(f.x, f.y), min(f.z, f.w)));
+    if (need <= here) {
+      __threadfence_block();
+      return here;
+    }
+    if ((it & 4095) == 0 && __any_sync(0xffffffffu, wait_over(st, t0, spin_ns, 102))) return 0x7fffffff;
+  }
+}
+
+// Barrier w + 1 belongs to warp w (0 is __syncthreads).  The warp converges
+// first: a barrier counts whole warps each time it is executed.
+__device__ __forceinline__ void bar_wait(int id, int threads) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  __syncwarp();
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// End of a step: the barriers its head names (n of them from that of warp w).
+struct StepEnd {
+  int n, bar, threads;
+  __device__ __forceinline__ explicit StepEnd(int sync)
+      : n(sync >> 14 & 15), bar((sync >> 10 & 15) + 1), threads(sync >> 18 & 1023) {}
+  __device__ __forceinline__ void arrive(int nwarp) const {
+    __syncwarp();
+    if (n > 0) asm volatile("bar.arrive %0, %1;" ::"r"(bar), "r"(threads) : "memory");
+    if (__builtin_expect(n > 1, 0))
+      for (int i = 1, w = bar; i < n; i++) {
+        w = w == nwarp ? 1 : w + 1;
+        asm volatile("bar.arrive %0, %1;" ::"r"(w), "r"(threads) : "memory");
+      }
+  }
+};
+
+__device__ __forceinline__ void report_end(Shared &sh, int step) {
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence_block();
+    sts(smem_addr(&sh.fin[step & 63]), step + 1);
+  }
+}
+
+// One triangular solve of the calling CTA: rows [b0, b0 + rows) of z or c0.
+// The window, from the start of dynamic shared memory: `rows` own results,
+// the zero, the halo.  The solves are inlined and read the problem's pointers
+// where they are used (from the constant bank, the descriptor being a kernel
+// parameter): copies of them, or a call, cost registers or reloads inside
+// the loop (measured on a chain of single rows: 0.53 against 0.81 ms).
+template <bool LOWER, typename T>
+__device__ __forceinline__ const TriSteps<T> &steps_of(const Dev<T> &D) {
+  if constexpr (LOWER) return D.SL;
+  else return D.SU;
+}
+
+template <typename T>
+__device__ __forceinline__ void steps_begin(const Dev<T> &D, Shared &sh) {
+  if (threadIdx.x < COPY_WARPS) sh.arrived[threadIdx.x] = 32 * threadIdx.x;  // first value of its share
+  if (threadIdx.x < 64) sh.fin[threadIdx.x] = 0;
+  if (threadIdx.x == 0) reinterpret_cast<T *>(nle_dyn_smem)[D.bsize * D.steps] = T(0);
+  __syncthreads();
+}
+
+// The copying warps of a step solve.
+template <bool LOWER, typename T>
+__device__ __forceinline__ void steps_copy(const Dev<T> &D, Shared &sh, long long spin_ns) {
+  const int m = (int)(threadIdx.x >> 5) - (NWARP - COPY_WARPS);
+  if (m < 0) return;
+  const TriSteps<T> &M = steps_of<LOWER>(D);
+  const int h0 = __ldg(M.hptr + grank()), h1 = __ldg(M.hptr + grank() + 1);
+  copy_halo<T>(M.hpos + h0, h1 - h0, m, LOWER ? D.z : D.c0,
+               smem_addr(nle_dyn_smem) + (unsigned)((D.bsize * D.steps + 1) * (int)sizeof(T)), sh, spin_ns, D.st);
+}
+
+// keeps the computation of a register where it is written: the compiler moves
+// loads, selects and address sums down to their first use otherwise, behind
+// the barrier that begins a step
+__device__ __forceinline__ void pin(unsigned &v) { asm volatile("" : "+r"(v)); }
+__device__ __forceinline__ void pin(float &v) { asm volatile("" : "+f"(v)); }
+__device__ __forceinline__ void pin(double &v) { asm volatile("" : "+d"(v)); }
+
+// two FP32 operations per instruction, each rounded as the single one
+using F2 = float2;
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 d;
+  asm("{.reg .b64 x, y, z, w;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmov.b64 z, {%6, %7};\n"
+      "fma.rn.f32x2 w, x, y, z;\nmov.b64 {%0, %1}, w;}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 d;
+  asm("{.reg .b64 x, y, w;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmul.rn.f32x2 w, x, y;\nmov.b64 {%0, %1}, w;}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 d;
+  asm("{.reg .b64 x, y, w;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nadd.rn.f32x2 w, x, y;\nmov.b64 {%0, %1}, w;}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+
+// Partial sums of a lane: NP of them, entry e of the lane in sum e mod NP.
+template <typename T, int NP>
+struct Sums;
+template <>
+struct Sums<float, 8> {
+  F2 acc[4];
+  template <int E>
+  __device__ __forceinline__ void start(const float (&a)[E], const float (&v)[E]) {
+#pragma unroll
+    for (int j = 0; j < 4; j++) acc[j] = mul2(F2{a[2 * j], a[2 * j + 1]}, F2{v[2 * j], v[2 * j + 1]});
+#pragma unroll
+    for (int e = 8; e < E; e += 2) acc[e / 2 & 3] = fma2(F2{a[e], a[e + 1]}, F2{v[e], v[e + 1]}, acc[e / 2 & 3]);
+  }
+  // the lane's quad i
+  __device__ __forceinline__ void quad(int i, const float (&a)[4], const float (&v)[4]) {
+#pragma unroll
+    for (int e = 0; e < 4; e += 2) {
+      const F2 x{a[e], a[e + 1]}, y{v[e], v[e + 1]};
+      if (i & 1) acc[2 + e / 2] = fma2(x, y, acc[2 + e / 2]);
+      else acc[e / 2] = fma2(x, y, acc[e / 2]);
+    }
+  }
+  __device__ __forceinline__ float total() const {
+    const F2 s = add2(add2(acc[0], acc[2]), add2(acc[1], acc[3]));
+    return s.x + s.y;
+  }
+};
+template <>
+struct Sums<double, 2> {
+  double acc[2];
+  template <int E>
+  __device__ __forceinline__ void start(const double (&a)[E], const double (&v)[E]) {
+    acc[0] = a[0] * v[0];
+    acc[1] = a[1] * v[1];
+#pragma unroll
+    for (int e = 2; e < E; e++) acc[e & 1] += a[e] * v[e];
+  }
+  __device__ __forceinline__ void quad(int, const double (&a)[4], const double (&v)[4]) {
+#pragma unroll
+    for (int e = 0; e < 4; e++) acc[e & 1] += a[e] * v[e];
+  }
+  __device__ __forceinline__ double total() const { return acc[0] + acc[1]; }
+};
+
+// LPR lanes per row, E entries of a lane held in registers (2 or quads; all of
+// them are summed, padding too: a predicated FP64 instruction costs as much).
+template <bool LOWER, int LPR, int E, typename T>
+__device__ __forceinline__ void trsv_steps(const Dev<T> &D, const T *rhs_all, Shared &sh, long long spin_ns) {
+  constexpr int PER = 32 / LPR, NP = sizeof(T) == 8 ? 2 : 8, C = E < 4 ? E : 4;
+  constexpr unsigned TS = sizeof(T);
+  const int64_t b0 = (int64_t)grank() * D.bsize * D.steps;
+  if (b0 >= D.npad) return;  // a CTA past the last solve slab
+  const TriSteps<T> &M = steps_of<LOWER>(D);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned w0 = smem_addr(nle_dyn_smem), zero = w0 + TS * (unsigned)(D.bsize * D.steps);
+  steps_begin(D, sh);
+  if (warp < D.step_warps) {
+    const int s0 = __ldg(M.step0 + grank()), ns = __ldg(M.step0 + grank() + 1) - s0;
+    const int4 *heads = reinterpret_cast<const int4 *>(M.head + s0);
+    const int32_t *rows = M.row + (int64_t)s0 * PER + lane / LPR;
+    const int nwarp = D.step_warps, next = warp + 1 == nwarp ? 1 : warp + 2;
+    const T *rhs = rhs_all + b0, *rdiag = D.rdiag + b0;
+    T *x = (LOWER ? D.z : D.c0) + b0;
+    unsigned c[E], own = 0;
+    T a[E], b = T(0), rdg = T(1);
+    int rl = 0;
+    auto head = [&](int t) { return t < ns ? __ldg(heads + 2 * t) : make_int4(0, 0, 0, 0); };
+    auto row_of = [&](int t) { return t < ns ? __ldg(rows + t * PER) : 0; };
+    // lanes past the step's repeat its last row (and store the same result)
+    auto lane_of = [&](int lanes) {
+      return LPR == 1 ? min(lane, lanes - 1) : lane < lanes ? lane : lanes - LPR + (lane & (LPR - 1));
+    };
+    // the step's coefficients, operands, right-hand side and pivot
+    auto fetch = [&](const int4 &H, int row) {
+      rl = row;
+      const int lanes = H.z & 63, n = H.z >> 6 & 1023;
+      const int32_t *po = M.opnd + 4 * ((int64_t)H.x + lane_of(lanes));
+      const T *pv = M.val + 4 * ((int64_t)H.x + lane_of(lanes));
+#pragma unroll
+      for (int i = 0; i < E; i += C) {
+        int ci[C] = {};
+        T ai[C] = {};
+        if (i < n) {
+          ldr(po + i * lanes, ci);
+          ldr(pv + i * lanes, ai);
+        }
+#pragma unroll
+        for (int e = 0; e < C; e++) c[i + e] = i < n ? w0 + (unsigned)ci[e] : zero, a[i + e] = ai[e];
+      }
+      rdg = __ldg(rdiag + rl);
+      b = __ldcg(rhs + rl);
+      own = w0 + TS * rl;
+      // all of it is in registers before the warp waits for its turn
+#pragma unroll
+      for (int e = 0; e < E; e++) pin(c[e]), pin(a[e]);
+      pin(rdg), pin(b), pin(own);
+    };
+    int t = warp;
+    // heads and rows two turns ahead, so that a fetch waits for one load only
+    int4 H = head(t), N = head(t + nwarp);
+    int nrow = row_of(t + nwarp);
+    if (t < ns) fetch(H, row_of(t));
+    int here = 0;  // halo values known to have arrived
+    for (; t < ns; t += nwarp) {
+      const unsigned flags = (unsigned)H.z >> 16;
+      const int n = H.z >> 6 & 1023, threads = H.y & 1023;
+      const bool plain = flags == 0 && n <= E;  // nothing special, all entries in registers
+      const StepEnd end(H.y);
+      __syncwarp();
+      if (H.w > here) here = await_halo(sh, H.w, spin_ns, D.st);
+      if (threads) bar_wait(warp + 1, threads);
+      if (__builtin_expect(!plain, 0)) {
+        if ((flags & STEP_EARLY) && nwarp > 1) bar_arrive(next, 64);
+        if (flags & STEP_WAIT) {
+          const int4 H2 = __ldg(heads + 2 * t + 1);
+          await_steps(sh, H2.y, H2.x - 1, spin_ns, D.st);
+        }
+      }
+      T v[E];
+#pragma unroll
+      for (int e = 0; e < E; e++) lds(c[e], v[e]);
+      Sums<T, NP> S;
+      S.start(a, v);
+      if (__builtin_expect(!plain, 0)) {
+        const int lanes = H.z & 63;
+#pragma unroll 1
+        for (int i = E / 4; 4 * i < n; i++) {  // quads past the ones in registers
+          const int64_t at = 4 * ((int64_t)H.x + lane_of(lanes) + (int64_t)i * lanes);
+          int ci[4];
+          T ai[4], vi[4];
+          ldr(M.opnd + at, ci);
+          ldr(M.val + at, ai);
+#pragma unroll
+          for (int e = 0; e < 4; e++) lds(w0 + (unsigned)ci[e], vi[e]);
+          S.quad(i, ai, vi);
+        }
+      }
+      T sum = S.total();
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      const T val = (b - sum) * rdg;
+      sts(own, val);
+      end.arrive(nwarp);
+      st_relaxed(x + rl, val);
+      if (flags & STEP_REPORT) {
+        __syncwarp();
+        report_end(sh, t);
+      }
+      H = N;
+      if (t + nwarp < ns) fetch(H, nrow);
+      N = head(t + 2 * nwarp);
+      nrow = row_of(t + 2 * nwarp);
+    }
+  }
+  steps_copy<LOWER>(D, sh, spin_ns);
+  __syncthreads();
+}
+
+// The step form of the forward (LOWER) or backward solve with right-hand side
+// rhs (global memory).
+template <bool LOWER, typename T>
+__device__ __forceinline__ void steps_solve(const Dev<T> &D, Shared &sh, const Ctl &ctl, const T *rhs) {
+  if constexpr (sizeof(T) == 8) {
+    if (D.step_n <= 2) trsv_steps<LOWER, 4, 2, T>(D, rhs, sh, ctl.spin_ns);
+    else trsv_steps<LOWER, 4, 4, T>(D, rhs, sh, ctl.spin_ns);
+  } else if (D.trows == 2) {
+    if (D.step_n <= 16) trsv_steps<LOWER, 2, 16, T>(D, rhs, sh, ctl.spin_ns);
+    else trsv_steps<LOWER, 2, 24, T>(D, rhs, sh, ctl.spin_ns);
+  } else {
+    if (D.step_n <= 8) trsv_steps<LOWER, 1, 8, T>(D, rhs, sh, ctl.spin_ns);
+    else trsv_steps<LOWER, 1, 16, T>(D, rhs, sh, ctl.spin_ns);
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ bool trsv_forward(const Dev<T> &D, Shared &sh, Ctl &ctl, int k) {
+  if constexpr (!kChainTU) {
+    if (D.steps) {
+      if (k == 0) {
+        steps_solve<true, T>(D, sh, ctl, D.g);
+        return true;
+      }
+      // w = g - R a (in y, which holds nothing needed any more)
+      constexpr int W = VT<T>::W;
+      const int64_t TT = gthreads();
+      for (int64_t ch = gtid(); ch < D.nchunks; ch += TT) {
+        T w[W];
+        ldc(D.g + ch * W, w);
+        for (int t = 0; t < k; t++) {
+          T r[W];
+          ldc(D.R + (int64_t)sh.order[t] * D.npad + ch * W, r);
+#pragma unroll
+          for (int v = 0; v < W; v++) w[v] -= T(sh.a[t]) * r[v];
+        }
+        stv(D.y + ch * W, w);
+      }
+      if (!grid_sync(D.st, sh, ctl, 20)) return false;
+      steps_solve<true, T>(D, sh, ctl, D.y);
+      return true;
+    }
+  }
   const TriEll<T> L{D.Loff, D.Lw, D.Lcol, D.Lval, D.rdiag, D.Lround, D.trows};
   T *bufA = reinterpret_cast<T *>(nle_dyn_smem);
   T *bufB = bufA + D.bsize;
@@ -252,13 +698,21 @@ __device__ __forceinline__ void trsv_forward(const Dev<T> &D, Shared &sh, const 
     trsv_block<true, T>(L, D.z, D.npad, D.bsize, ctl.twarps, ctl.spin_ns, ctl.poll_ns, D.st, bufA,
                         [&](int64_t r) { return bufB[r - b0]; });
   }
+  return true;
 }
 
 // The right-hand side of the backward solve is the forward result of the
-// CTA's own slab (buffer A), complete after trsv_forward's closing
-// __syncthreads, so no grid barrier separates the two solves.
+// CTA's own slab (buffer A, or z in the step form), complete after
+// trsv_forward's closing __syncthreads, so no grid barrier separates the two
+// solves.
 template <typename T>
-__device__ __forceinline__ void trsv_backward(const Dev<T> &D, const Ctl &ctl) {
+__device__ __forceinline__ void trsv_backward(const Dev<T> &D, Shared &sh, const Ctl &ctl) {
+  if constexpr (!kChainTU) {
+    if (D.steps) {
+      steps_solve<false, T>(D, sh, ctl, D.z);
+      return;
+    }
+  }
   const TriEll<T> U{D.Uoff, D.Uw, D.Ucol, D.Uval, D.rdiag, D.Uround, D.trows};
   const T *bufA = reinterpret_cast<const T *>(nle_dyn_smem);
   T *bufB = reinterpret_cast<T *>(nle_dyn_smem) + D.bsize;
@@ -286,9 +740,9 @@ __device__ bool precond_tail(const Dev<T> &D, Shared &sh, Ctl &ctl, int m, int k
                              bool use_beta, double *gamma_new) {
   constexpr int W = VT<T>::W;
   const int64_t tid = gtid(), TT = gthreads();
-  trsv_forward<T>(D, sh, ctl, k);
+  if (!trsv_forward<T>(D, sh, ctl, k)) return false;
   tmark(sh, PH_FWD);
-  trsv_backward<T>(D, ctl);
+  trsv_backward<T>(D, sh, ctl);
   if (!grid_sync(D.st, sh, ctl, 21)) return false;
   tmark(sh, PH_BWD);
   // dot products of c0: slots [0,k) r_t^T c0 ; k: g^T c0 ; [k+1, k+1+m) q_c^T c0
@@ -410,10 +864,7 @@ __device__ bool pcg_solve(const Dev<T> &D, const Opts &O, Shared &sh, Ctl &ctl, 
   if (threadIdx.x == 0)
     for (int s = 0; s < k; s++) sh.sg[s] = sh.sc[1 + s];
   __syncthreads();
-  coef_a(sh, k);
-  double gamma;
-  if (!precond_tail<T, RPC>(D, sh, ctl, m, k, D.p, 0.0, false, &gamma)) return false;
-
+  double gamma = 0.0;
   res.g0 = g0;
   res.gn = g0;
   res.eres = 0.0;
@@ -422,6 +873,14 @@ __device__ bool pcg_solve(const Dev<T> &D, const Opts &O, Shared &sh, Ctl &ctl, 
   res.its = 0;
   double gprev = g0, eprev = 0.0;
   for (int l = 0; l < max_pcg; l++) {
+    // direction p = P_k g + beta p (one copy of the solves' code for the first
+    // direction and the others)
+    coef_a(sh, k);
+    {
+      double gnew;
+      if (!precond_tail<T, RPC>(D, sh, ctl, m, k, D.p, gamma, l > 0, &gnew)) return false;
+      gamma = gnew;
+    }
     // --- pass A: y = (A - theta I) p, delta = p^T y, Q^T y
     T yv[RPC][W];
     {
@@ -537,10 +996,6 @@ __device__ bool pcg_solve(const Dev<T> &D, const Opts &O, Shared &sh, Ctl &ctl, 
     if (threadIdx.x == 0)
       for (int s = 0; s < k; s++) sh.sg[s] = sh.sc[4 + s];
     __syncthreads();
-    coef_a(sh, k);
-    double gnew;
-    if (!precond_tail<T, RPC>(D, sh, ctl, m, k, D.p, gamma, true, &gnew)) return false;
-    gamma = gnew;
     gprev = gn;
     eprev = eres;
   }

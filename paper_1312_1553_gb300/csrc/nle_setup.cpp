@@ -420,18 +420,142 @@ static void ell(int64_t n, int64_t npad, int64_t bsize, bool lower, const std::v
 }
 
 template <typename TV>
-void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S) {
+void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S, bool with_ell) {
   pack<TV>(P.n, P.npad, H, P.Arp, P.Acol, P.Aval, 0, 0, S.A);
   pack<double>(P.n, P.npad, H, P.Arp, P.Acol, P.Aval, 0, 0, S.A64);
   const std::vector<int32_t> *lev = level_rounds ? &P.lev : nullptr;
-  ell<TV>(P.n, P.npad, bsize, true, P.Lrp, P.Lcol, P.Lval, lev, R, S.L);
-  ell<TV>(P.n, P.npad, bsize, false, P.Urp, P.Ucol, P.Uval, lev, R, S.U);
+  if (with_ell) {
+    ell<TV>(P.n, P.npad, bsize, true, P.Lrp, P.Lcol, P.Lval, lev, R, S.L);
+    ell<TV>(P.n, P.npad, bsize, false, P.Urp, P.Ucol, P.Uval, lev, R, S.U);
+  }
   S.diag.assign(P.npad, TV(1));
   for (int64_t i = 0; i < P.n; i++) S.diag[i] = TV(1.0 / P.diag[i]);  // reciprocal pivots
 }
 
-template void build_sell<float>(const Permuted &, int, int64_t, bool, int, SellSet<float> &);
-template void build_sell<double>(const Permuted &, int, int64_t, bool, int, SellSet<double> &);
+template void build_sell<float>(const Permuted &, int, int64_t, bool, int, SellSet<float> &, bool);
+template void build_sell<double>(const Permuted &, int, int64_t, bool, int, SellSet<double> &, bool);
+
+template <typename TV>
+void plan_steps(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps, StepsHost<TV> &out) {
+  const int64_t n = P.n, ns = (P.npad + rows - 1) / rows, per = 32 / lpr;
+  const std::vector<int64_t> &rp = lower ? P.Lrp : P.Urp;
+  const std::vector<int32_t> &col = lower ? P.Lcol : P.Ucol;
+  std::vector<int64_t> seen(n, -1);  // last solve slab that listed the position
+  out.step0.assign(ns + 1, 0);
+  out.hptr.assign(ns + 1, 0);
+  out.head.clear();
+  out.row.clear();
+  out.hpos.clear();
+  out.halo_max = 0;
+  out.n_max = 0;
+  int64_t off = 0;
+  std::vector<int32_t> order;
+  std::vector<int64_t> start;
+  for (int64_t s = 0; s < ns; s++) {
+    const int64_t b0 = s * rows, b1 = std::min(P.npad, b0 + rows), nb = b1 - b0;
+    // rows by level (counting sort, stable), padding rows as a level of
+    // their own behind the others; reversed for L^T
+    auto lev = [&](int64_t i) -> int64_t { return b0 + i < n ? P.lev[b0 + i] : -1; };
+    int64_t lmin = INT32_MAX, lmax = -1;
+    for (int64_t i = 0; i < nb; i++)
+      if (lev(i) >= 0) lmin = std::min(lmin, lev(i)), lmax = std::max(lmax, lev(i));
+    if (lmax < 0) lmin = 0;
+    auto key = [&](int64_t i) { return lev(i) < 0 ? lmax + 1 - lmin : lev(i) - lmin; };
+    start.assign(lmax - lmin + 3, 0);
+    for (int64_t i = 0; i < nb; i++) start[key(i) + 1]++;
+    for (size_t k = 1; k < start.size(); k++) start[k] += start[k - 1];
+    order.resize(nb);
+    for (int64_t i = 0; i < nb; i++) order[start[key(i)]++] = (int32_t)i;
+    if (!lower) std::reverse(order.begin(), order.end());
+    int32_t t = 0, prev = 0, nprev = 0;  // step; first step of the level before, its steps
+    for (int64_t i0 = 0; i0 < nb;) {
+      int64_t i1 = i0 + 1;
+      while (i1 < nb && key(order[i1]) == key(order[i0])) i1++;
+      const int32_t first = t, nst = (int32_t)((i1 - i0 + per - 1) / per);
+      const bool many = nst > nwarps - 1, manyprev = nprev > nwarps - 1;
+      int64_t i2 = i1;  // the level behind this one: its steps
+      while (i2 < nb && key(order[i2]) == key(order[i1])) i2++;
+      const int32_t nnext = (int32_t)((i2 - i1 + per - 1) / per);
+      const bool direct = nst + nnext <= nwarps, directprev = nprev > 0 && nprev + nst <= nwarps;
+      for (int32_t u = 0; u < nst; u++, t++) {
+        const int64_t a = i0 + u * per, e = std::min(i1, a + per);
+        int64_t w = 0;
+        for (int64_t i = a; i < a + per; i++) {
+          out.row.push_back(order[std::min(i, e - 1)]);
+          const int64_t r = b0 + order[std::min(i, e - 1)];
+          if (i >= e || r >= n) continue;
+          w = std::max(w, rp[r + 1] - rp[r]);
+          for (int64_t k = rp[r]; k < rp[r + 1]; k++) {
+            const int32_t c = col[k];
+            if ((c < b0 || c >= b1) && seen[c] != s) {
+              seen[c] = s;
+              out.hpos.push_back(c);
+            }
+          }
+        }
+        const int64_t lanes = (e - a) * lpr, wl = (w + lpr - 1) / lpr, q = (wl + 3) / 4;
+        const bool last = u + 1 == nst;
+        // the slab's first level waits for nothing
+        const uint32_t flags = (many ? STEP_REPORT : 0) | (last || directprev || first == 0 ? 0 : STEP_EARLY) |
+                               (manyprev ? STEP_WAIT : 0);
+        uint32_t sync = 0;
+        if (nwarps > 1 && first > 0) sync = u > 0 && !directprev ? 64 : 32 * (1 + (manyprev ? 1 : nprev));
+        if (nwarps > 1 && nnext && (last || !many))
+          sync |= (uint32_t)((first + nst) % nwarps) << 10 | (uint32_t)(direct ? nnext : 1) << 14 |
+                  (uint32_t)(32 * (1 + (many ? 1 : nst))) << 18;
+        out.head.push_back({(int32_t)(off / 4), sync, (uint32_t)(lanes | (wl << 6) | (flags << 16)),
+                            (int32_t)((int64_t)out.hpos.size() - out.hptr[s]), first, prev, {0, 0}});
+        off += 4 * q * lanes;
+        out.n_max = std::max(out.n_max, (int)wl);
+      }
+      nprev = nst;
+      prev = first;
+      i0 = i1;
+    }
+    out.step0[s + 1] = (int32_t)out.head.size();
+    out.hptr[s + 1] = (int32_t)out.hpos.size();
+    out.halo_max = std::max<int64_t>(out.halo_max, out.hptr[s + 1] - out.hptr[s]);
+  }
+  out.opnd.resize(off);
+  out.val.resize(off);
+}
+
+template <typename TV>
+void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost<TV> &out) {
+  const int64_t n = P.n, ns = (P.npad + rows - 1) / rows, per = 32 / lpr;
+  const std::vector<int64_t> &rp = lower ? P.Lrp : P.Urp;
+  const std::vector<int32_t> &col = lower ? P.Lcol : P.Ucol;
+  const std::vector<double> &val = lower ? P.Lval : P.Uval;
+  const int64_t ts = (int64_t)sizeof(TV);
+  std::vector<int32_t> slot(n, 0);  // window slot of the solve slab's halo values
+  std::fill(out.opnd.begin(), out.opnd.end(), (int32_t)(rows * ts));
+  std::fill(out.val.begin(), out.val.end(), TV(0));
+  for (int64_t s = 0; s < ns; s++) {
+    const int64_t b0 = s * rows, b1 = std::min(P.npad, b0 + rows);
+    for (int32_t h = out.hptr[s]; h < out.hptr[s + 1]; h++) slot[out.hpos[h]] = (int32_t)(rows + 1 + h - out.hptr[s]);
+    for (int32_t t = out.step0[s]; t < out.step0[s + 1]; t++) {
+      const StepHead &H = out.head[t];
+      const int64_t lanes = H.shape & 63;
+      for (int64_t u = 0; u < lanes / lpr; u++) {
+        const int64_t r = b0 + out.row[t * per + u];
+        if (r >= n) continue;
+        for (int64_t e = rp[r]; e < rp[r + 1]; e++) {
+          const int64_t k = e - rp[r], m = k / lpr, c = col[e];
+          const int64_t at = 4 * ((int64_t)H.off + (m / 4) * lanes + u * lpr + k % lpr) + m % 4;
+          out.opnd[at] = (int32_t)((c >= b0 && c < b1 ? c - b0 : slot[c]) * ts);
+          out.val[at] = TV(val[e]);
+        }
+      }
+    }
+  }
+}
+
+#define NLE_STEPS(TV)                                                                              \
+  template void plan_steps<TV>(const Permuted &, int64_t, bool, int, int, StepsHost<TV> &);       \
+  template void build_steps<TV>(const Permuted &, int64_t, bool, int, StepsHost<TV> &);
+NLE_STEPS(float)
+NLE_STEPS(double)
+#undef NLE_STEPS
 
 template <typename TV>
 void build_chain(const Permuted &P, int64_t bsize, bool lower, int nwarps, ChainHost<TV> &out) {

@@ -4,6 +4,8 @@
 #include <string>
 #include <vector>
 
+#include "nle_internal.h"
+
 namespace nle {
 
 struct Factor {
@@ -50,6 +52,36 @@ struct EllHost {
   // steps (entries past the 2 * 32 / R a warp step prefetches, in steps of
   // 32 / R; 255: up to the slab's width)
   std::vector<uint16_t> round;
+};
+
+// Steps of one strictly triangular factor.  The rows of each solve slab (some
+// consecutive slabs) are sorted by level, then position (the other way round
+// for L^T), and cut at every change of level and after every 32 / lpr rows (lpr
+// lanes per row).  An operand is the offset of its value in the solve slab's
+// shared-memory window: its own results, a slot that holds 0, and its halo
+// (the values of other solve slabs, in the order in which the steps first
+// need them).
+// Entry k of a row belongs to lane k % lpr of the row and is that lane's entry
+// number k / lpr; a lane's entries come in quads of four, padded with zeros,
+// and a step stores quad after quad, lane after lane.
+// Steps that follow each other belong to consecutive ones of nwarps warps.
+// Where the warps of two consecutive levels are all different, every step of
+// the second starts with a barrier of its warp and of all warps of the first.
+// Elsewhere the first step of a level starts with a barrier of its warp and
+// of all warps of the level before (of that level's last step only, with
+// STEP_WAIT, if these are too many), and each step releases the next one of
+// its level (STEP_EARLY).
+template <typename TV>
+struct StepsHost {
+  std::vector<int32_t> step0;  // per solve slab + 1: first step
+  std::vector<StepHead> head;  // per step
+  std::vector<int32_t> row;    // 32 / lpr per step: rows, relative to the solve slab
+  std::vector<int32_t> opnd;   // operands, in bytes from the start of the CTA's dynamic shared memory
+  std::vector<TV> val;         // coefficients, same order
+  std::vector<int32_t> hptr;   // per solve slab + 1: first halo value
+  std::vector<int32_t> hpos;   // position of every halo value
+  int64_t halo_max = 0;        // largest halo of a solve slab
+  int n_max = 0;               // most entries of a lane
 };
 
 // Chain schedule of one strictly triangular factor (see trsv_chain): the
@@ -108,7 +140,18 @@ void permute(int64_t n, const int64_t *rp, const int32_t *ci, const double *va, 
 // schedule takes at a time, 4 or 2) into one round per level (needed when
 // dependencies can point to later slabs; see trsv_block).
 template <typename TV>
-void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S);
+void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S,
+                bool with_ell = true);
+
+// Steps of the strictly lower (lower = true) or upper factor for solve slabs of
+// `rows` rows, with lpr (1, 2, 4 or 8) lanes per row and nwarps warps.
+// plan_steps cuts the steps and collects the halo of every solve slab;
+// build_steps then fills in operands and coefficients for a window of own
+// results from element 0, the zero at element `rows` and the halo behind it.
+template <typename TV>
+void plan_steps(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps, StepsHost<TV> &out);
+template <typename TV>
+void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost<TV> &out);
 
 // Chain schedule of the strictly lower (lower = true: P.Lrp/Lcol/Lval, levels
 // P.lev) or upper (P.Urp/Ucol/Uval, levels P.levU) factor for nwarps warps
