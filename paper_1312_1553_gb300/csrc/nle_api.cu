@@ -464,7 +464,7 @@ static nle_status get_vector(nle_t h, const T *src, double *dst, int on_device) 
 // lists; 0: slab-major level-minor order with level rounds), uploaded on the
 // handle's stream.  rp/ci/va: the matrix that was factored.
 template <typename TV>
-static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, int chain) {
+static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, int chain, bool with_a) {
   const int H = 32 * h->vw;
   SellSet<TV> S;
   // step form of the level schedule where the window of a solve slab (own
@@ -479,8 +479,9 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
     h->step_warps = std::max(1, std::min(STEP_WARPS, h->opt.trsv_warps));
     for (int m = solve_slabs(h, P); m >= 1; m /= 2) {
       h->halo_n = h->step_n = 0;
+      both([&] { plan_steps<TV>(P, h->bsize * m, true, lpr, h->step_warps, G[0]); },
+           [&] { plan_steps<TV>(P, h->bsize * m, false, lpr, h->step_warps, G[1]); });
       for (int d = 0; d < 2; d++) {
-        plan_steps<TV>(P, h->bsize * m, d == 0, lpr, h->step_warps, G[d]);
         h->halo_n = (int)std::max<int64_t>(h->halo_n, G[d].halo_max);
         h->step_n = std::max(h->step_n, G[d].n_max);
       }
@@ -489,17 +490,23 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
       h->steps = 0;
     }
   }
-  build_sell<TV>(P, H, h->bsize, level_rounds, h->trows, S, !h->steps);
-  NLE_CUDA(h, upload(h->A_sptr, S.A.sptr, h->stream));
-  NLE_CUDA(h, upload(h->A_col, S.A.col, h->stream));
-  NLE_CUDA(h, upload(h->A_val, S.A.val, h->stream));
-  NLE_CUDA(h, upload(h->A64_val, S.A64.val, h->stream));
-  NLE_CUDA(h, upload(h->d_diag, S.diag, h->stream));
+  both([&] { build_sell<TV>(P, H, h->bsize, level_rounds, h->trows, S, !h->steps && !chain, with_a); },
+       [&] {
+         if (h->steps)
+           both([&] { build_steps<TV>(P, h->bsize * h->steps, true, lpr, G[0]); },
+                [&] { build_steps<TV>(P, h->bsize * h->steps, false, lpr, G[1]); });
+       });
+  if (with_a) {
+    NLE_CUDA(h, upload(h->A_sptr, S.A.sptr, h->stream));
+    NLE_CUDA(h, upload(h->A_col, S.A.col, h->stream));
+    NLE_CUDA(h, upload(h->A_val, S.A.val, h->stream));
+    NLE_CUDA(h, upload(h->A64_val, S.A64.val, h->stream));
+    NLE_CUDA(h, upload(h->d_diag, S.diag, h->stream));
+  }
   if (chain) {
     const int nw = std::max(1, std::min(NWARP, h->opt.trsv_warps));
     ChainHost<TV> CL, CU;
-    build_chain<TV>(P, h->bsize, true, nw, CL);
-    build_chain<TV>(P, h->bsize, false, nw, CU);
+    both([&] { build_chain<TV>(P, h->bsize, true, nw, CL); }, [&] { build_chain<TV>(P, h->bsize, false, nw, CU); });
     h->nstrands = CL.nstrands;
     S.L = std::move(CL.ell);
     S.U = std::move(CU.ell);
@@ -512,8 +519,7 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
   }
   if (h->steps) {
     for (int d = 0; d < 2; d++) {
-      StepsHost<TV> &g = G[d];
-      build_steps<TV>(P, h->bsize * h->steps, d == 0, lpr, g);
+      const StepsHost<TV> &g = G[d];
       NLE_CUDA(h, upload(h->step_buf[d][0], g.step0, h->stream));
       NLE_CUDA(h, upload(h->step_buf[d][1], g.head, h->stream));
       NLE_CUDA(h, upload(h->step_buf[d][2], g.row, h->stream));
@@ -539,31 +545,41 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
   return NLE_OK;
 }
 
+// kept: the relabelled matrix of the level candidates.  While it is in place
+// (n set), A and the numbering on the device are of this relabelling and only
+// the triangular layout is built; a chain layout replaces both and clears it.
 static nle_status build_layout(nle_t h, const std::vector<int32_t> &P0, const int64_t *rp, const int32_t *ci,
-                               const double *va, int chain, int trows = TRSV_ROWS) {
+                               const double *va, int chain, int trows, Permuted &kept) {
   h->trows = chain ? TRSV_ROWS : trows;
+  const bool fresh = chain || kept.n == 0;
   if (chain) {
+    kept.n = 0;
     h->perm.resize(h->n);
     h->iperm.resize(h->n);
     for (int64_t i = 0; i < h->n; i++) h->perm[i] = h->iperm[i] = (int32_t)i;
-  } else {
+  } else if (fresh) {
     // with a multicolour ordering the slabs still follow the caller's row
     // order (P0[k] = caller's row of row k of P A P^T), which keeps each
     // slab's rows and their neighbours together
     slab_level_order(h->F, h->bsize, P0.empty() ? nullptr : P0.data(), h->perm, h->iperm);
   }
-  Permuted P;
-  permute(h->n, rp, ci, va, h->F, h->perm, h->iperm, h->npad, P);
-  if (!P0.empty()) {
-    // device position -> row of the caller's numbering, through P A P^T
-    for (int64_t p = 0; p < h->n; p++) h->perm[p] = P0[h->perm[p]];
-    for (int64_t p = 0; p < h->n; p++) h->iperm[h->perm[p]] = (int32_t)p;
+  Permuted own;
+  Permuted &P = chain ? own : kept;
+  if (fresh) {
+    permute(h->n, rp, ci, va, h->F, h->perm, h->iperm, h->npad, P);
+    if (!P0.empty()) {
+      // device position -> row of the caller's numbering, through P A P^T
+      for (int64_t p = 0; p < h->n; p++) h->perm[p] = P0[h->perm[p]];
+      for (int64_t p = 0; p < h->n; p++) h->iperm[h->perm[p]] = (int32_t)p;
+    }
   }
-  nle_status s = mixed(h) ? upload_layout<float>(h, P, !P0.empty(), chain)
-                          : upload_layout<double>(h, P, !P0.empty(), chain);
+  nle_status s = mixed(h) ? upload_layout<float>(h, P, !P0.empty(), chain, fresh)
+                          : upload_layout<double>(h, P, !P0.empty(), chain, fresh);
   if (s != NLE_OK) return s;
-  NLE_CUDA(h, upload(h->d_perm, h->perm, h->stream));
-  NLE_CUDA(h, upload(h->d_iperm, h->iperm, h->stream));
+  if (fresh) {
+    NLE_CUDA(h, upload(h->d_perm, h->perm, h->stream));
+    NLE_CUDA(h, upload(h->d_iperm, h->iperm, h->stream));
+  }
   h->chain = chain;
   return NLE_OK;
 }
@@ -895,26 +911,31 @@ nle_status nle_factor_ic(nle_t h, int lfil, double tau_ic) {
     return fail(h, NLE_ERR_ARG, "the chain schedule needs the natural ordering");
   h->tune_ms[0] = h->tune_ms[1] = h->tune_ms[2] = 0.0;
   const int rows_opt = h->opt.trsv_rows;
+  Permuted kept;
   if (sched == NLE_SCHED_AUTO) {
     struct Cand {
       int chain, rows, slot;
     };
+    // level with 4 rows last: it is the usual winner, whose layout is then in
+    // place, and the level candidates share the relabelling and A (the
+    // 7-point 64^3 in mixed precision, with L and U built on two threads:
+    // 465 -> 239 ms)
     std::vector<Cand> cands;
-    if (rows_opt == 0 || rows_opt == 4) cands.push_back({0, 4, 0});
     if (chain_ok) cands.push_back({1, TRSV_ROWS, 1});
     if (rows_opt == 0 || rows_opt == 2) cands.push_back({0, 2, 2});
+    if (rows_opt == 0 || rows_opt == 4) cands.push_back({0, 4, 0});
     int best = -1;
     for (size_t c = 0; c < cands.size(); c++) {
-      if ((s = build_layout(h, P0, rp, ci, va, cands[c].chain, cands[c].rows)) != NLE_OK) return s;
+      if ((s = build_layout(h, P0, rp, ci, va, cands[c].chain, cands[c].rows, kept)) != NLE_OK) return s;
       if ((s = time_precond(h, &h->tune_ms[cands[c].slot])) != NLE_OK) return s;
       if (best < 0 || h->tune_ms[cands[c].slot] < h->tune_ms[cands[best].slot]) best = (int)c;
     }
     // the last candidate's layout is in place; rebuild the fastest one
     if (best != (int)cands.size() - 1 &&
-        (s = build_layout(h, P0, rp, ci, va, cands[best].chain, cands[best].rows)) != NLE_OK)
+        (s = build_layout(h, P0, rp, ci, va, cands[best].chain, cands[best].rows, kept)) != NLE_OK)
       return s;
   } else {
-    if ((s = build_layout(h, P0, rp, ci, va, sched == NLE_SCHED_CHAIN ? 1 : 0, rows_opt == 2 ? 2 : 4)) != NLE_OK)
+    if ((s = build_layout(h, P0, rp, ci, va, sched == NLE_SCHED_CHAIN ? 1 : 0, rows_opt == 2 ? 2 : 4, kept)) != NLE_OK)
       return s;
   }
   NLE_CUDA(h, cudaStreamSynchronize(h->stream));

@@ -295,17 +295,23 @@ void permute_csr(int64_t n, const int64_t *rp, const int32_t *ci, const double *
 void slab_level_order(const Factor &F, int64_t bsize, const int32_t *locality, std::vector<int32_t> &perm,
                       std::vector<int32_t> &iperm) {
   const int64_t n = F.n;
+  auto loc = [&](int64_t r) -> int64_t { return locality ? locality[r] : r; };
+  // every slab holds bsize consecutive locality values, so ordering by
+  // (slab, level, locality) fills each slab's position range exactly.  Two
+  // stable counting passes over the rows taken by locality: first by level,
+  // then by slab.
+  std::vector<int32_t> by(n);
+  for (int64_t i = 0; i < n; i++) by[loc(i)] = (int32_t)i;
+  std::vector<int64_t> at(F.nlevL + 1, 0);
   perm.resize(n);
-  for (int64_t i = 0; i < n; i++) perm[i] = (int32_t)i;
-  auto loc = [&](int32_t r) -> int64_t { return locality ? locality[r] : r; };
-  // every slab holds bsize consecutive locality values, so sorting by
-  // (slab, level, locality) fills each slab's position range exactly
-  std::sort(perm.begin(), perm.end(), [&](int32_t a, int32_t b) {
-    const int64_t sa = loc(a) / bsize, sb = loc(b) / bsize;
-    if (sa != sb) return sa < sb;
-    if (F.levL[a] != F.levL[b]) return F.levL[a] < F.levL[b];
-    return loc(a) < loc(b);
-  });
+  for (int64_t i = 0; i < n; i++) at[F.levL[i] + 1]++;
+  for (int64_t l = 0; l < F.nlevL; l++) at[l + 1] += at[l];
+  for (int64_t i = 0; i < n; i++) perm[at[F.levL[by[i]]]++] = by[i];
+  by.swap(perm);
+  const int64_t ns = (n + bsize - 1) / bsize;
+  at.resize(ns);
+  for (int64_t s = 0; s < ns; s++) at[s] = s * bsize;
+  for (int64_t i = 0; i < n; i++) perm[at[loc(by[i]) / bsize]++] = by[i];
   iperm.assign(n, 0);
   for (int64_t p = 0; p < n; p++) iperm[perm[p]] = (int32_t)p;
 }
@@ -420,20 +426,23 @@ static void ell(int64_t n, int64_t npad, int64_t bsize, bool lower, const std::v
 }
 
 template <typename TV>
-void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S, bool with_ell) {
-  pack<TV>(P.n, P.npad, H, P.Arp, P.Acol, P.Aval, 0, 0, S.A);
-  pack<double>(P.n, P.npad, H, P.Arp, P.Acol, P.Aval, 0, 0, S.A64);
+void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S, bool with_ell,
+                bool with_a) {
+  if (with_a) {
+    pack<TV>(P.n, P.npad, H, P.Arp, P.Acol, P.Aval, 0, 0, S.A);
+    pack<double>(P.n, P.npad, H, P.Arp, P.Acol, P.Aval, 0, 0, S.A64);
+    S.diag.assign(P.npad, TV(1));
+    for (int64_t i = 0; i < P.n; i++) S.diag[i] = TV(1.0 / P.diag[i]);  // reciprocal pivots
+  }
   const std::vector<int32_t> *lev = level_rounds ? &P.lev : nullptr;
   if (with_ell) {
     ell<TV>(P.n, P.npad, bsize, true, P.Lrp, P.Lcol, P.Lval, lev, R, S.L);
     ell<TV>(P.n, P.npad, bsize, false, P.Urp, P.Ucol, P.Uval, lev, R, S.U);
   }
-  S.diag.assign(P.npad, TV(1));
-  for (int64_t i = 0; i < P.n; i++) S.diag[i] = TV(1.0 / P.diag[i]);  // reciprocal pivots
 }
 
-template void build_sell<float>(const Permuted &, int, int64_t, bool, int, SellSet<float> &, bool);
-template void build_sell<double>(const Permuted &, int, int64_t, bool, int, SellSet<double> &, bool);
+template void build_sell<float>(const Permuted &, int, int64_t, bool, int, SellSet<float> &, bool, bool);
+template void build_sell<double>(const Permuted &, int, int64_t, bool, int, SellSet<double> &, bool, bool);
 
 template <typename TV>
 void plan_steps(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps, StepsHost<TV> &out) {
@@ -733,59 +742,68 @@ void permute(int64_t n, const int64_t *rp, const int32_t *ci, const double *va, 
     P.lev[i] = F.levL[perm[i]];
     P.levU[i] = F.levU[perm[i]];
   }
-  // A' = P A P^T, rows sorted by new column
-  std::vector<std::pair<int32_t, double>> tmp;
-  P.Arp.assign(n + 1, 0);
-  P.Acol.clear();
-  P.Aval.clear();
-  P.Acol.reserve(rp[n]);
-  P.Aval.reserve(rp[n]);
-  for (int64_t i = 0; i < n; i++) {
-    const int64_t o = perm[i];
-    tmp.clear();
-    for (int64_t e = rp[o]; e < rp[o + 1]; e++) tmp.push_back({iperm[ci[e]], va[e]});
-    std::sort(tmp.begin(), tmp.end(), [](auto &a, auto &b) { return a.first < b.first; });
-    for (auto &t : tmp) {
-      P.Acol.push_back(t.first);
-      P.Aval.push_back(t.second);
+  auto matrix = [&] {
+    std::vector<std::pair<int32_t, double>> tmp;
+    // A' = P A P^T, rows sorted by new column
+    P.Arp.assign(n + 1, 0);
+    P.Acol.clear();
+    P.Aval.clear();
+    P.Acol.reserve(rp[n]);
+    P.Aval.reserve(rp[n]);
+    for (int64_t i = 0; i < n; i++) {
+      const int64_t o = perm[i];
+      tmp.clear();
+      for (int64_t e = rp[o]; e < rp[o + 1]; e++) tmp.push_back({iperm[ci[e]], va[e]});
+      std::sort(tmp.begin(), tmp.end(), [](auto &a, auto &b) { return a.first < b.first; });
+      for (auto &t : tmp) {
+        P.Acol.push_back(t.first);
+        P.Aval.push_back(t.second);
+      }
+      P.Arp[i + 1] = (int64_t)P.Acol.size();
     }
-    P.Arp[i + 1] = (int64_t)P.Acol.size();
-  }
-  // strictly lower part of L' and strictly upper part of U' = L'^T, diagonal
-  P.diag.assign(n, 0.0);
-  P.Lrp.assign(n + 1, 0);
-  P.Lcol.clear();
-  P.Lval.clear();
-  for (int64_t i = 0; i < n; i++) {
-    const int64_t o = perm[i];
-    tmp.clear();
-    for (int64_t e = F.Lrowptr[o]; e < F.Lrowptr[o + 1]; e++) {
-      if (F.Lcol[e] == o)
-        P.diag[i] = F.Lval[e];
-      else
-        tmp.push_back({iperm[F.Lcol[e]], F.Lval[e]});
+  };
+  auto lower = [&] {
+    std::vector<std::pair<int32_t, double>> tmp;
+    // strictly lower part of L' and strictly upper part of U' = L'^T, diagonal
+    P.diag.assign(n, 0.0);
+    P.Lrp.assign(n + 1, 0);
+    P.Lcol.clear();
+    P.Lval.clear();
+    for (int64_t i = 0; i < n; i++) {
+      const int64_t o = perm[i];
+      tmp.clear();
+      for (int64_t e = F.Lrowptr[o]; e < F.Lrowptr[o + 1]; e++) {
+        if (F.Lcol[e] == o)
+          P.diag[i] = F.Lval[e];
+        else
+          tmp.push_back({iperm[F.Lcol[e]], F.Lval[e]});
+      }
+      std::sort(tmp.begin(), tmp.end(), [](auto &a, auto &b) { return a.first < b.first; });
+      for (auto &t : tmp) {
+        P.Lcol.push_back(t.first);
+        P.Lval.push_back(t.second);
+      }
+      P.Lrp[i + 1] = (int64_t)P.Lcol.size();
     }
-    std::sort(tmp.begin(), tmp.end(), [](auto &a, auto &b) { return a.first < b.first; });
-    for (auto &t : tmp) {
-      P.Lcol.push_back(t.first);
-      P.Lval.push_back(t.second);
+  };
+  auto upper = [&] {
+    std::vector<std::pair<int32_t, double>> tmp;
+    P.Urp.assign(n + 1, 0);
+    P.Ucol.clear();
+    P.Uval.clear();
+    for (int64_t i = 0; i < n; i++) {
+      const int64_t o = perm[i];  // row i of U' = column o of L
+      tmp.clear();
+      for (int64_t e = F.Ccolptr[o] + 1; e < F.Ccolptr[o + 1]; e++) tmp.push_back({iperm[F.Crow[e]], F.Cval[e]});
+      std::sort(tmp.begin(), tmp.end(), [](auto &a, auto &b) { return a.first < b.first; });
+      for (auto &t : tmp) {
+        P.Ucol.push_back(t.first);
+        P.Uval.push_back(t.second);
+      }
+      P.Urp[i + 1] = (int64_t)P.Ucol.size();
     }
-    P.Lrp[i + 1] = (int64_t)P.Lcol.size();
-  }
-  P.Urp.assign(n + 1, 0);
-  P.Ucol.clear();
-  P.Uval.clear();
-  for (int64_t i = 0; i < n; i++) {
-    const int64_t o = perm[i];  // row i of U' = column o of L
-    tmp.clear();
-    for (int64_t e = F.Ccolptr[o] + 1; e < F.Ccolptr[o + 1]; e++) tmp.push_back({iperm[F.Crow[e]], F.Cval[e]});
-    std::sort(tmp.begin(), tmp.end(), [](auto &a, auto &b) { return a.first < b.first; });
-    for (auto &t : tmp) {
-      P.Ucol.push_back(t.first);
-      P.Uval.push_back(t.second);
-    }
-    P.Urp[i + 1] = (int64_t)P.Ucol.size();
-  }
+  };
+  both(matrix, [&] { both(lower, upper); });
 }
 
 }  // namespace nle

@@ -2,6 +2,8 @@
 #pragma once
 #include <cstdint>
 #include <string>
+#include <future>
+#include <system_error>
 #include <vector>
 
 #include "nle_internal.h"
@@ -141,7 +143,21 @@ void permute(int64_t n, const int64_t *rp, const int32_t *ci, const double *va, 
 // dependencies can point to later slabs; see trsv_block).
 template <typename TV>
 void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S,
-                bool with_ell = true);
+                bool with_ell = true, bool with_a = true);
+
+// Run a and b, a on a thread of its own where one can be had.  An exception of
+// either leaves only after both have ended.
+template <typename FA, typename FB>
+void both(FA a, FB b) {
+  std::future<void> f;
+  try {
+    f = std::async(std::launch::async, [&a] { a(); });
+  } catch (const std::system_error &) {
+    a();
+  }
+  b();
+  if (f.valid()) f.get();
+}
 
 // Steps of the strictly lower (lower = true) or upper factor for solve slabs of
 // `rows` rows, with lpr (1, 2, 4 or 8) lanes per row and nwarps warps.
