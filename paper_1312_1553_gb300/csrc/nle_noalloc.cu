@@ -7,6 +7,7 @@
 // the runtime for the array's device address once per device.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstdio>
 #include <mutex>
@@ -36,45 +37,125 @@ __global__ void k_na_fill(double *z, double *c, int64_t n, int *err) {
   if (blockIdx.x == 0 && threadIdx.x == 0) *err = 0;
 }
 
-// One warp per row, rows taken round-robin in order (ascending for the lower
-// factor, descending for the upper one): a row only waits for rows owned by
-// other warps that are resident (cooperative launch), so every wait ends.
-// Entries whose column is not strictly below (above) the row, or outside
-// [0, n), are skipped and reported; every wait is bounded.
+constexpr int kWarps = 32;  // warps of a CTA
+constexpr int kRows = 4;    // rows a warp has open at a time, 32 / kRows lanes each
+constexpr int kLanes = 32 / kRows;
+constexpr int kSleep = 40;  // ns between two rounds of looks that found nothing
+
+// Quotient t / d given inv = 1 / d rounded: one corrected product where its
+// steps can neither overflow nor lose bits, the division otherwise.  Three
+// dependent FP64 instructions after t is known instead of the division's
+// dozen.
+__device__ __forceinline__ double quotient(double t, double d, double inv) {
+  const double q = t * inv;
+  const unsigned eq = ((unsigned)__double2hiint(q) >> 20) & 0x7ff, ed = ((unsigned)__double2hiint(d) >> 20) & 0x7ff;
+  if (eq - (1023u - 498u) > 996u || ed - (1023u - 332u) > 664u) return t / d;
+  return fma(fma(-q, d, t), inv, q);
+}
+
+// Four rows per warp, eight lanes a row and two entries of a lane in flight;
+// groups of four rows are taken round-robin in order (ascending for the lower
+// factor, descending for the upper one).  A row waits only for rows of earlier
+// groups and for earlier rows of its own.  The warps are all resident
+// (cooperative launch), and a warp looks at the missing values of all its
+// rows in turn without stopping at one, so every wait ends.  Entries whose
+// column is not strictly below (above) the row, or outside [0, n), are skipped
+// and reported; every wait is bounded.
+//
+// Bound by the latency of one dependency (store, look through L2, sum) times
+// the number of dependencies in a line that the rows in flight cannot overlap.
+// So many rows are open at a time (32 warps an SM x 4: 19,456, nine planes of
+// a 45 x 50 x 55 grid), and what does not depend on the
+// solution (pointers, coefficients, right-hand side, reciprocal pivot) is read
+// before the first look.  A lane adds its entries in order and eight lanes
+// meet in a tree: the sum does not depend on when values arrive.
+// Both solves together, against one warp per row that divided after the last
+// value arrived and read its row after the row before was done (1,216 rows in
+// flight): n = 123,750 7-point 28.7 -> 1.39 ms.  With 8 and 16 warps an SM
+// 5.39 and 2.89 ms, with 2 rows a warp (16 lanes each) 3.28, with 8 rows 1.60
+// (2.65 against 2.52 on 300 x 350 5-point, 1.91 against 2.34 on 27-point
+// 40^3); no pause, 40 ns and 200 ns between looks 1.39, 1.39, 1.41.
 template <bool LOWER>
-__global__ void __launch_bounds__(256) k_na_solve(int64_t n, const int32_t *rp, const int32_t *col,
-                                                  const double *val, const double *diag, const double *rhs,
-                                                  double *x, int *err, long long lim_cycles) {
-  const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(32 * kWarps) k_na_solve(int64_t n, const int32_t *rp, const int32_t *col,
+                                                          const double *val, const double *diag, const double *rhs,
+                                                          double *x, int *err, long long lim_cycles) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31, sub = lane % kLanes;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t it = w; it < n; it += nw) {
+  for (int64_t g = w; g * kRows < n; g += nw) {
+    const int64_t it = g * kRows + lane / kLanes;
     const int64_t r = LOWER ? it : n - 1 - it;
-    const int e0 = __ldg(rp + r), e1 = __ldg(rp + r + 1);
-    double acc = 0.0;
-    for (int e = e0 + lane; e < e1; e += 32) {
-      const int64_t c = __ldg(col + e);
-      const bool ok = LOWER ? (c >= 0 && c < r) : (c > r && c < n);
-      if (!ok) {
-        atomicCAS(err, 0, (int)NLE_ERR_CSR);
-        continue;
-      }
-      double xv = nle::ld_relaxed(x + c);
-      if (nle::is_sent(xv)) {
-        const long long c0 = clock64();
-        while (nle::is_sent(xv)) {
-          xv = nle::ld_relaxed(x + c);
-          if (nle::is_sent(xv) && clock64() - c0 > lim_cycles) {
-            atomicCAS(err, 0, (int)NLE_ERR_TIMEOUT);
-            xv = 0.0;
-          }
+    bool open = it < n;  // the row has not been published
+    int e = 0, e1 = 0;
+    double b = 0.0, d = 1.0;
+    if (open) {
+      e = __ldg(rp + r) + sub;
+      e1 = __ldg(rp + r + 1);
+      b = __ldg(rhs + r);
+      d = __ldg(diag + r);
+    }
+    int c[2];
+    double v[2], xv[2];
+    bool miss[2];
+    auto fetch = [&] {
+#pragma unroll
+      for (int t = 0; t < 2; t++) {
+        const int k = e + t * kLanes;
+        c[t] = k < e1 ? __ldg(col + k) : 0;
+        v[t] = k < e1 ? __ldg(val + k) : 0.0;
+        xv[t] = 0.0;
+        miss[t] = k < e1;
+        if (miss[t] && !(LOWER ? (c[t] >= 0 && c[t] < r) : (c[t] > r && c[t] < n))) {
+          atomicCAS(err, 0, (int)NLE_ERR_CSR);
+          v[t] = 0.0;
+          miss[t] = false;
         }
       }
-      acc += __ldg(val + e) * xv;
-    }
+    };
+    fetch();
+    const double inv = 1.0 / d;
+    double acc = 0.0;
+    long long c0 = clock64();
+    while (true) {
+      if (miss[0]) xv[0] = nle::ld_relaxed(x + c[0]);
+      if (miss[1]) xv[1] = nle::ld_relaxed(x + c[1]);
+      miss[0] = miss[0] && nle::is_sent(xv[0]);
+      miss[1] = miss[1] && nle::is_sent(xv[1]);
+      bool moved = e < e1 && !miss[0] && !miss[1];
+      if (moved) {
+        acc += v[0] * xv[0];
+        acc += v[1] * xv[1];
+        e += 2 * kLanes;
+        if (e < e1) fetch();
+      }
+      const unsigned ready = __ballot_sync(kFull, e >= e1);
+      const bool publish = open && ((ready >> (lane - sub)) & ((1u << kLanes) - 1)) == (1u << kLanes) - 1;
+      if (__any_sync(kFull, publish)) {
+        double s = acc;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) nle::st_relaxed(x + r, (__ldg(rhs + r) - acc) / __ldg(diag + r));
+        for (int o = kLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        if (publish && sub == 0) nle::st_relaxed(x + r, quotient(b - s, d, inv));
+        if (publish) open = false;
+        if (!__any_sync(kFull, open)) break;
+        moved = true;
+      }
+      if (__any_sync(kFull, moved)) {
+        c0 = clock64();
+      } else {
+        if (clock64() - c0 > lim_cycles) {
+          // nothing came for this warp: report, and go on with zeros
+#pragma unroll
+          for (int t = 0; t < 2; t++)
+            if (miss[t]) {
+              atomicCAS(err, 0, (int)NLE_ERR_TIMEOUT);
+              xv[t] = 0.0;
+              miss[t] = false;
+            }
+        }
+        __nanosleep(kSleep);
+      }
+    }
   }
 }
 
@@ -147,6 +228,7 @@ extern "C" nle_status nle_ic_apply_noalloc(int64_t n, const int32_t *Lrp, const 
   (void)cudaGetLastError();
   k_na_fill<<<256, 256, 0, s>>>(z, c, n, err);
   e = cudaGetLastError();
+  const int grid = (int)std::min<int64_t>(nsm, (n + kWarps * kRows - 1) / (kWarps * kRows));
   int64_t nn = n;
   const double *zc = z;
   void *fa[] = {&nn, (void *)&Lrp, (void *)&Lcol, (void *)&Lval, (void *)&diag, (void *)&g, (void *)&z, (void *)&err,
@@ -154,9 +236,9 @@ extern "C" nle_status nle_ic_apply_noalloc(int64_t n, const int32_t *Lrp, const 
   void *ba[] = {&nn, (void *)&Urp, (void *)&Ucol, (void *)&Uval, (void *)&diag, (void *)&zc, (void *)&c, (void *)&err,
                 (void *)&lim};
   if (e == cudaSuccess)
-    e = cudaLaunchCooperativeKernel((void *)k_na_solve<true>, dim3(nsm), dim3(256), fa, 0, s);
+    e = cudaLaunchCooperativeKernel((void *)k_na_solve<true>, dim3(grid), dim3(32 * kWarps), fa, 0, s);
   if (e == cudaSuccess)
-    e = cudaLaunchCooperativeKernel((void *)k_na_solve<false>, dim3(nsm), dim3(256), ba, 0, s);
+    e = cudaLaunchCooperativeKernel((void *)k_na_solve<false>, dim3(grid), dim3(32 * kWarps), ba, 0, s);
   int herr = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
