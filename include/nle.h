@@ -97,13 +97,15 @@ typedef struct {
   int dacg_recompute;    /* recompute A x in DACG every this many iterations (default 50) */
   double spin_timeout_s; /* bound on each device-side wait, seconds (default 2.0) */
   int grid_ctas;         /* persistent grid size; 0 = one CTA per SM (default 0) */
-  int trsv_warps;        /* warps per CTA in the triangular solves, 1..16 (default 16) */
+  int trsv_warps;        /* warps per CTA in the triangular solves, 1..16 (default 16); the step
+                            form of the level schedule takes at most 12, beside 4 that copy */
   int ordering;          /* NLE_ORDER_NATURAL (default) or a multicolour ordering, see
                             nle_multicolor_order; applied before the IC factor */
   int bfgs_update;       /* NLE_BFGS_SIMPLIFIED (default) or NLE_BFGS_FULL */
   int trsv_schedule;     /* NLE_SCHED_AUTO (default), NLE_SCHED_LEVEL or NLE_SCHED_CHAIN */
   int trsv_poll_ns;      /* pause (ns, 0..10000) a warp of the triangular solves takes between
-                            two polls of inputs that are not ready (default 0: none) */
+                            two polls of inputs that are not ready (default 0: none); the step
+                            form's warps wait at barriers and take no pause */
   int trsv_rows;         /* level schedule: rows a warp takes at a time, 4 (8 lanes per row)
                             or 2 (16 lanes, for factors with wide rows); 0 (default): chosen
                             by the autotuner under NLE_SCHED_AUTO, 4 otherwise */
@@ -132,8 +134,14 @@ typedef struct {
  * Both give the same solution (up to rounding order); they differ in how
  * the rows are dealt to the GPU's warps:
  *   NLE_SCHED_LEVEL  rows of each CTA's slab sorted by level of L, groups
- *                    of 4 rows per warp step, every row polling its own
- *                    inputs (no barrier between levels);
+ *                    of 4 (2) rows per warp step.  Step form, where the slab
+ *                    and the values it needs of other slabs fit in shared
+ *                    memory: the warps take a level's steps in turn and hand
+ *                    over through barriers, four more copy in the other
+ *                    slabs' values as they appear.  Polled form otherwise,
+ *                    and for FP64 with 2 rows: every row polls its own
+ *                    inputs, no barrier between levels.  Both forms give the same
+ *                    bits;
  *   NLE_SCHED_CHAIN  the factored matrix's own row order; runs of rows in
  *                    which each row depends on its predecessor (the grid
  *                    lines of a stencil matrix in natural order) stay on one

@@ -57,20 +57,48 @@ void *kernel_ptr<double>(int id, int rpc, int chain) {
   return nullptr;
 }
 
-// ---------------------------------------------------------------------------
-// relabelling kernels
-// ---------------------------------------------------------------------------
-// dst[i] = T(src[perm[i]]) for i < n, 0 for n <= i < npad
+// dst[c*npad + i] = T(src[c*n + perm[i]]) for i < n, 0 in the padding, column
+// c = blockIdx.y.  Bound by the latency of two dependent loads: a thread has
+// four rows in flight (a warp's rows are consecutive, so perm and dst are
+// whole lines), and all columns go in one launch, one after the other so that the
+// lines of a column that neighbouring slabs share are still in L2.  One row in
+// flight and one launch per column before: a preconditioner call of 16
+// columns, n = 10^6, 1.52 -> 1.41 ms, n = 4,200 325 -> 308 us (with one wait for
+// the stream less).
+constexpr int MOVE_ROWS = 4, MOVE_TPB = 256;
+static unsigned move_blocks(int64_t rows) { return (unsigned)((rows + MOVE_ROWS * MOVE_TPB - 1) / (MOVE_ROWS * MOVE_TPB)); }
 template <typename T>
-__global__ void k_gather(T *dst, const double *src, const int32_t *perm, int64_t n, int64_t npad) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npad; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = (i < n) ? T(src[perm[i]]) : T(0);
+__global__ void __launch_bounds__(MOVE_TPB) k_gather(T *dst, const double *src, const int32_t *perm, int64_t n,
+                                                     int64_t npad) {
+  const int64_t i0 = (int64_t)blockIdx.x * (MOVE_ROWS * MOVE_TPB) + threadIdx.x;
+  src += blockIdx.y * n;
+  dst += blockIdx.y * npad;
+  int32_t from[MOVE_ROWS];
+  double v[MOVE_ROWS];
+#pragma unroll
+  for (int u = 0; u < MOVE_ROWS; u++) from[u] = i0 + u * MOVE_TPB < n ? __ldg(perm + i0 + u * MOVE_TPB) : -1;
+#pragma unroll
+  for (int u = 0; u < MOVE_ROWS; u++) v[u] = from[u] >= 0 ? src[from[u]] : 0.0;
+#pragma unroll
+  for (int u = 0; u < MOVE_ROWS; u++)
+    if (i0 + u * MOVE_TPB < npad) dst[i0 + u * MOVE_TPB] = T(v[u]);
 }
-// dst[o] = double(src[iperm[o]]) for o < n
+// dst[o] = double(src[iperm[o]]) for o < n, unless st is given and the work
+// before it on the stream has recorded an error there.  Rows in flight as above.
 template <typename T>
-__global__ void k_scatter(double *dst, const T *src, const int32_t *iperm, int64_t n) {
-  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < n; o += (int64_t)gridDim.x * blockDim.x)
-    dst[o] = double(src[iperm[o]]);
+__global__ void __launch_bounds__(MOVE_TPB) k_scatter(double *dst, const T *src, const int32_t *iperm, int64_t n,
+                                                      const State *st) {
+  if (st && st->err != 0) return;
+  const int64_t o0 = (int64_t)blockIdx.x * (MOVE_ROWS * MOVE_TPB) + threadIdx.x;
+  int32_t from[MOVE_ROWS];
+  T v[MOVE_ROWS];
+#pragma unroll
+  for (int u = 0; u < MOVE_ROWS; u++) from[u] = o0 + u * MOVE_TPB < n ? __ldg(iperm + o0 + u * MOVE_TPB) : 0;
+#pragma unroll
+  for (int u = 0; u < MOVE_ROWS; u++) v[u] = src[from[u]];
+#pragma unroll
+  for (int u = 0; u < MOVE_ROWS; u++)
+    if (o0 + u * MOVE_TPB < n) dst[o0 + u * MOVE_TPB] = double(v[u]);
 }
 // V[j*n + o] = sgn_j * Qt[j*npad + iperm[o]], sgn_j making the entry of
 // largest modulus positive (lowest natural index on ties).  One block per j.
@@ -432,29 +460,43 @@ static nle_status ensure_q(nle_t h, int m) {
   return NLE_OK;
 }
 
-// Copy p vectors of length n (natural order, FP64, host or device) into a
-// device array of working-precision columns (device order) at dst + c*npad.
+// Copy count vectors of length n (natural order, FP64, host or device) into a
+// device array of working-precision columns (device order) at dst + c*npad:
+// one launch for device vectors, one per column through the staging buffer
+// for host vectors.
 template <typename T>
 static nle_status put_vectors(nle_t h, const double *src, int count, T *dst, int on_device) {
   const int64_t n = h->n;
-  for (int c = 0; c < count; c++) {
+  const int step = on_device ? count : 1;
+  for (int c = 0; c < count; c += step) {
     const double *s = src + (int64_t)c * n;
     if (!on_device) {
       NLE_CUDA(h, cudaMemcpyAsync(h->scratch.p, s, n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
       s = h->scratch.as<double>();
     }
-    k_gather<T><<<1024, 256, 0, h->stream>>>(dst + (int64_t)c * h->npad, s, h->d_perm.as<int32_t>(), n, h->npad);
+    k_gather<T><<<dim3(move_blocks(h->npad), step), MOVE_TPB, 0, h->stream>>>(dst + (int64_t)c * h->npad, s,
+                                                                             h->d_perm.as<int32_t>(), n, h->npad);
     NLE_CUDA(h, cudaGetLastError());
   }
   return NLE_OK;
 }
 
+// Close a call whose kernel is on the stream: report its error, or give its
+// result src (device order) to dst (natural order, FP64).  dst is not written
+// after an error.  A device dst is filled before the error is known on the
+// host (the copy kernel looks itself), so the call waits for the stream once.
+// check = false for kernels without waits, which record no errors.
 template <typename T>
-static nle_status get_vector(nle_t h, const T *src, double *dst, int on_device) {
+static nle_status get_vector(nle_t h, const T *src, double *dst, int on_device, bool check = true) {
+  nle_status s = check && !on_device ? check_state_error(h) : NLE_OK;
+  if (s != NLE_OK) return s;
   double *d = on_device ? dst : h->scratch.as<double>();
-  k_scatter<T><<<1024, 256, 0, h->stream>>>(d, src, h->d_iperm.as<int32_t>(), h->n);
+  k_scatter<T><<<move_blocks(h->n), MOVE_TPB, 0, h->stream>>>(d, src, h->d_iperm.as<int32_t>(), h->n,
+                                                             check ? h->state.as<State>() : nullptr);
   NLE_CUDA(h, cudaGetLastError());
+  if (on_device && check) return check_state_error(h);
   if (!on_device) NLE_CUDA(h, cudaMemcpyAsync(dst, d, h->n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  NLE_CUDA(h, cudaStreamSynchronize(h->stream));
   return NLE_OK;
 }
 
@@ -592,7 +634,8 @@ static nle_status time_precond_t(nle_t h, double *ms) {
   Dev<T> D = make_dev<T>(h);
   k_default_start<<<1024, 256, 0, h->stream>>>(h->scratch.as<double>(), h->n, 0);
   NLE_CUDA(h, cudaGetLastError());
-  k_gather<T><<<1024, 256, 0, h->stream>>>(D.g, h->scratch.as<double>(), h->d_perm.as<int32_t>(), h->n, h->npad);
+  k_gather<T><<<move_blocks(h->npad), MOVE_TPB, 0, h->stream>>>(D.g, h->scratch.as<double>(), h->d_perm.as<int32_t>(), h->n,
+                                                             h->npad);
   NLE_CUDA(h, cudaGetLastError());
   Opts O = make_opts(h, 1e-8, 1, 1);
   // the timing runs are the library's own: their waits are bounded by at
@@ -1112,10 +1155,7 @@ static nle_status shifted_impl(nle_t h, double theta, const double *x, double *y
   void *fn = kernel_ptr<T>(K_SHIFTED, h->rpc, h->chain);
   void *args[] = {&D, &theta};
   NLE_CUDA(h, cudaLaunchKernel(fn, dim3(h->grid), dim3(TPB), args, 0, h->stream));
-  s = get_vector<T>(h, D.y, y, on_dev);
-  if (s != NLE_OK) return s;
-  NLE_CUDA(h, cudaStreamSynchronize(h->stream));
-  return NLE_OK;
+  return get_vector<T>(h, D.y, y, on_dev, false);
 }
 
 extern "C" nle_status nle_apply_shifted(nle_t h, double theta, const double *x, double *y, int buffers_on_device) {
@@ -1143,10 +1183,7 @@ static nle_status prec_impl(nle_t h, int k, const double *S, const double *R, in
   NLE_CUDA(h, cudaMemsetAsync(h->state.p, 0, sizeof(State), h->stream));
   void *args[] = {&D, &O, &m, &k};
   if ((s = launch<T>(h, K_PREC, args)) != NLE_OK) return s;
-  if ((s = check_state_error(h)) != NLE_OK) return s;
-  if ((s = get_vector<T>(h, D.y, c, on_dev)) != NLE_OK) return s;
-  NLE_CUDA(h, cudaStreamSynchronize(h->stream));
-  return NLE_OK;
+  return get_vector<T>(h, D.y, c, on_dev);
 }
 
 extern "C" nle_status nle_apply_prec(nle_t h, int k, const double *S, const double *R, int m, const double *Q,
@@ -1177,7 +1214,6 @@ static nle_status pcg_impl(nle_t h, double theta, double tol, int max_pcg, const
   NLE_CUDA(h, cudaMemsetAsync(h->state.p, 0, sizeof(State), h->stream));
   void *args[] = {&D, &O, &m, &k, &theta, &max_pcg};
   if ((s = launch<T>(h, K_PCG, args)) != NLE_OK) return s;
-  if ((s = check_state_error(h)) != NLE_OK) return s;
   if ((s = get_vector<T>(h, D.s, sout, on_dev)) != NLE_OK) return s;
   State st;
   NLE_CUDA(h, cudaMemcpyAsync(&st, h->state.p, sizeof(State), cudaMemcpyDeviceToHost, h->stream));
