@@ -603,7 +603,7 @@ __device__ __forceinline__ void trsv_steps(const Dev<T> &D, const T *rhs_all, Sh
       if (__builtin_expect(!plain, 0)) {
         const int lanes = H.z & 63;
 #pragma unroll 1
-        for (int i = E / 4; 4 * i < n; i++) {  // quads past the ones in registers
+        for (int i = (E + 3) / 4; 4 * i < n; i++) {  // quads past the ones in registers
           const int64_t at = 4 * ((int64_t)H.x + lane_of(lanes) + (int64_t)i * lanes);
           int ci[4];
           T ai[4], vi[4];
