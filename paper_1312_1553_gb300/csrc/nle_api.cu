@@ -523,6 +523,7 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
       h->halo_n = h->step_n = 0;
       both([&] { plan_steps<TV>(P, h->bsize * m, true, lpr, h->step_warps, G[0]); },
            [&] { plan_steps<TV>(P, h->bsize * m, false, lpr, h->step_warps, G[1]); });
+      if (!G[0].fits || !G[1].fits) break;
       for (int d = 0; d < 2; d++) {
         h->halo_n = (int)std::max<int64_t>(h->halo_n, G[d].halo_max);
         h->step_n = std::max(h->step_n, G[d].n_max);

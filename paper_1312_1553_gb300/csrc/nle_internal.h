@@ -64,6 +64,16 @@ constexpr uint32_t STEP_EARLY = 2;   // releases the next step, of the same leve
 constexpr uint32_t STEP_WAIT = 4;    // a level with reports before: waits for them
 constexpr int COPY_WARPS = 4;        // warps of a CTA that copy the halo
 constexpr int STEP_WARPS = NWARP - COPY_WARPS;  // most solving warps (one named barrier each)
+// Most entries of a lane: what StepHead states.  Longer rows (lfil bounds the
+// columns of L, not its rows) take the polled form.  Below that the step form is
+// the better one: one application, all rows of the level equally long, 64 hubs at a
+// time, rows of 96 / 384 / 1,020 entries, polled -> step form, FP64 77 / 385 / 3,345
+// -> 46 / 55 / 68 us, FP32 56 / 182 / 1,854 -> 36 / 49 / 78 us; one hub behind the
+// other FP64 346 / 1,182 / 3,342 -> 223 / 619 / 1,466 us, FP32 with two lanes 194 /
+// 446 / 1,853 -> 144 / 578 / 1,537 us.
+constexpr int STEP_N_MAX = 1023;
+static_assert(STEP_WARPS < 16 && 32 * (STEP_WARPS + 1) < 1024, "StepHead::sync: 4 bits a warp, 10 the threads of a barrier");
+static_assert(STEP_N_MAX < 1024, "StepHead::shape: 10 bits the entries of a lane");
 template <typename T>
 struct TriSteps {
   const int32_t *step0;  // per solve slab: first step

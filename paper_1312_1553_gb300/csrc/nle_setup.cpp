@@ -457,6 +457,12 @@ void plan_steps(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps
   out.hpos.clear();
   out.halo_max = 0;
   out.n_max = 0;
+  out.opnd.clear();
+  out.val.clear();
+  int64_t longest = 0;
+  for (int64_t r = 0; r < n; r++) longest = std::max(longest, rp[r + 1] - rp[r]);
+  out.fits = (longest + lpr - 1) / lpr <= STEP_N_MAX;
+  if (!out.fits) return;
   int64_t off = 0;
   std::vector<int32_t> order;
   std::vector<int64_t> start;
@@ -536,6 +542,7 @@ void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost
   const std::vector<int32_t> &col = lower ? P.Lcol : P.Ucol;
   const std::vector<double> &val = lower ? P.Lval : P.Uval;
   const int64_t ts = (int64_t)sizeof(TV);
+  if (!out.fits) return;
   std::vector<int32_t> slot(n, 0);  // window slot of the solve slab's halo values
   std::fill(out.opnd.begin(), out.opnd.end(), (int32_t)(rows * ts));
   std::fill(out.val.begin(), out.val.end(), TV(0));

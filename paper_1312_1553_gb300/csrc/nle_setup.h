@@ -84,6 +84,7 @@ struct StepsHost {
   std::vector<int32_t> hpos;   // position of every halo value
   int64_t halo_max = 0;        // largest halo of a solve slab
   int n_max = 0;               // most entries of a lane
+  bool fits = false;           // every lane has at most STEP_N_MAX entries; no steps otherwise
 };
 
 // Chain schedule of one strictly triangular factor (see trsv_chain): the
@@ -161,8 +162,8 @@ void both(FA a, FB b) {
 
 // Steps of the strictly lower (lower = true) or upper factor for solve slabs of
 // `rows` rows, with lpr (1, 2, 4 or 8) lanes per row and nwarps warps.
-// plan_steps cuts the steps and collects the halo of every solve slab;
-// build_steps then fills in operands and coefficients for a window of own
+// plan_steps cuts the steps and collects the halo of every solve slab, unless
+// a row is too long (out.fits = false, no steps); build_steps then fills in operands and coefficients for a window of own
 // results from element 0, the zero at element `rows` and the halo behind it.
 template <typename TV>
 void plan_steps(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps, StepsHost<TV> &out);
