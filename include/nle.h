@@ -141,7 +141,7 @@ typedef struct {
  *                    slabs' values as they appear.  Polled form otherwise,
  *                    and for FP64 with 2 rows: every row polls its own
  *                    inputs, no barrier between levels.  Both forms give the same
- *                    bits;
+ *                    bits (the sign of a zero aside);
  *   NLE_SCHED_CHAIN  the factored matrix's own row order; runs of rows in
  *                    which each row depends on its predecessor (the grid
  *                    lines of a stencil matrix in natural order) stay on one

@@ -282,7 +282,7 @@ constexpr bool kChainTU = NLE_CHAIN_TU != 0;
 // Sums are formed as the 8-lane (16-lane) reduction of trsv_block forms them:
 // entry k of a row in partial sum k mod 8 (16), each partial sum in ascending
 // k, the partial sums added pairwise in the order of its butterfly, so both
-// forms give the same bits.  With LPR lanes per row, lane g holds the partial
+// forms give the same bits (the sign of a zero aside).  With LPR lanes per row, lane g holds the partial
 // sums p with p mod LPR = g: the first additions are in the lane, the others
 // between lanes.  FP32: one (two) lanes, since a shuffle costs as much as six
 // additions.  FP64: four, since an FP64 instruction occupies its quarter of
@@ -520,21 +520,23 @@ struct Sums<float, 8> {
     return s.x + s.y;
   }
 };
+// Every FP64 product goes into an fma and every other sum is an explicit add: of two
+// products that meet in one sum the compiler picks the one it rounds, and rows of more
+// than 8 entries differed from trsv_block's in the last bit.
 template <>
 struct Sums<double, 2> {
   double acc[2];
   template <int E>
   __device__ __forceinline__ void start(const double (&a)[E], const double (&v)[E]) {
-    acc[0] = a[0] * v[0];
-    acc[1] = a[1] * v[1];
+    acc[0] = acc[1] = 0.0;
 #pragma unroll
-    for (int e = 2; e < E; e++) acc[e & 1] += a[e] * v[e];
+    for (int e = 0; e < E; e++) acc[e & 1] = fma(a[e], v[e], acc[e & 1]);
   }
   __device__ __forceinline__ void quad(int, const double (&a)[4], const double (&v)[4]) {
 #pragma unroll
-    for (int e = 0; e < 4; e++) acc[e & 1] += a[e] * v[e];
+    for (int e = 0; e < 4; e++) acc[e & 1] = fma(a[e], v[e], acc[e & 1]);
   }
-  __device__ __forceinline__ double total() const { return acc[0] + acc[1]; }
+  __device__ __forceinline__ double total() const { return __dadd_rn(acc[0], acc[1]); }
 };
 
 // LPR lanes per row, E entries of a lane held in registers (2 or quads; all of
