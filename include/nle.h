@@ -203,6 +203,8 @@ typedef struct {
   double ms_batch;              /* device time of the batched launch that solved this
                                    problem (nle_batch_solve; 0 after nle_solve) */
   int trsv_schedule;            /* NLE_SCHED_LEVEL or NLE_SCHED_CHAIN: the schedule in use */
+  int trsv_slabs;               /* level schedule, step form: slabs a CTA solves (1, 2 or 4); 0: polled
+                                   form, or chain schedule */
   double tune_ms_level;         /* autotuner: device ms of one (L L^T)^{-1} application with */
   double tune_ms_chain;         /*   each candidate (0 when not timed): level schedule with 4 */
   double tune_ms_level2;        /*   rows per warp step, chain schedule, level with 2 rows */

@@ -1042,6 +1042,7 @@ static void fill_stats(const State &st, int p, double ms_dacg, double ms_newton,
 // schedule of the handle's triangular solves and the autotuner's timings
 static void schedule_stats(nle_t h, nle_stats *stats) {
   stats->trsv_schedule = h->chain ? NLE_SCHED_CHAIN : NLE_SCHED_LEVEL;
+  stats->trsv_slabs = h->steps;
   stats->trsv_rows = h->trows;
   stats->tune_ms_level = h->tune_ms[0];
   stats->tune_ms_chain = h->tune_ms[1];

@@ -58,7 +58,8 @@ class nle_stats(ctypes.Structure):
                 ("pcg_iterations", ctypes.c_int64), ("pcg_sum_m", ctypes.c_int64), ("pcg_sum_k", ctypes.c_int64),
                 ("dacg_iterations", ctypes.c_int64), ("dacg_sum_m", ctypes.c_int64),
                 ("kernel_launches", ctypes.c_int64), ("ms_phase", ctypes.c_double * 8), ("ascending", ctypes.c_int),
-                ("ms_batch", ctypes.c_double), ("trsv_schedule", ctypes.c_int), ("tune_ms_level", ctypes.c_double),
+                ("ms_batch", ctypes.c_double), ("trsv_schedule", ctypes.c_int), ("trsv_slabs", ctypes.c_int),
+                ("tune_ms_level", ctypes.c_double),
                 ("tune_ms_chain", ctypes.c_double), ("tune_ms_level2", ctypes.c_double), ("strands", ctypes.c_int64),
                 ("trsv_rows", ctypes.c_int), ("ic_on_device", ctypes.c_int), ("ms_ic_factor", ctypes.c_double),
                 ("ms_ic_kernel", ctypes.c_double), ("ms_ic_setup", ctypes.c_double)]
@@ -378,6 +379,7 @@ def stats_dict(s: nle_stats) -> dict:
                 ms_batch=float(s.ms_batch), trsv_schedule=SCHEDULES.get(int(s.trsv_schedule), "none"),
                 tune_ms=dict(level=float(s.tune_ms_level), chain=float(s.tune_ms_chain),
                              level2=float(s.tune_ms_level2)), strands=int(s.strands), trsv_rows=int(s.trsv_rows),
+                trsv_slabs=int(s.trsv_slabs),
                 ic=dict(on_device=int(s.ic_on_device), factor_ms=float(s.ms_ic_factor),
                         kernel_ms=float(s.ms_ic_kernel), setup_ms=float(s.ms_ic_setup)))
 
