@@ -136,12 +136,14 @@ typedef struct {
  *   NLE_SCHED_LEVEL  rows of each CTA's slab sorted by level of L, groups
  *                    of 4 (2) rows per warp step.  Step form, where the slab
  *                    and the values it needs of other slabs fit in shared
- *                    memory: the warps take a level's steps in turn and hand
- *                    over through barriers, four more copy in the other
- *                    slabs' values as they appear.  Polled form otherwise,
- *                    and for FP64 with 2 rows: every row polls its own
- *                    inputs, no barrier between levels.  Both forms give the same
- *                    bits (the sign of a zero aside);
+ *                    memory, no row of L or L^T has more than 1,023 entries
+ *                    (2,046 with 2 rows, 4,092 in FP64) and nle_factor_ic
+ *                    forecasts it to be faster: the warps take a level's
+ *                    steps in turn and hand over through barriers, four more
+ *                    copy in the other slabs' values as they appear.  Polled
+ *                    form otherwise, and for FP64 with 2 rows: every row
+ *                    polls its own inputs, no barrier between levels.  Both
+ *                    forms give the same bits (the sign of a zero aside);
  *   NLE_SCHED_CHAIN  the factored matrix's own row order; runs of rows in
  *                    which each row depends on its predecessor (the grid
  *                    lines of a stencil matrix in natural order) stay on one

@@ -566,7 +566,79 @@ void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost
   }
 }
 
+// Costs in us, fitted to one application of (L L^T)^{-1} on 7-point (20^3 to
+// 106^3), 5-point, 27-point and random geometric graph factors, natural and both
+// multicolour orderings: the forecasts of 67 measured times each miss by 8 to
+// 15 % (root mean square).
+static FormCost form_cost(bool dbl, int lpr, int regs) {
+  if (dbl) return {regs <= 2 ? 0.36 : 0.41, 0.065, 0.80, 0.0030, 0.36, 0.63, 0.004, 0.38, 0.85, 0.47};
+  if (lpr == 2) return {0.16, 0.084, 0.65, 0.0033, 0.19, 0.29, 0.018, 0.71, 0.39, 0.29};
+  return {regs <= 8 ? 0.086 : 0.146, 0.12, 0.65, 0.0034, 0.20, 0.29, 0.022, 0.63, 0.25, 0.40};
+}
+
+template <typename TV>
+Forecast forecast(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps, int twarps,
+                  const StepsHost<TV> &plan) {
+  // entries of a lane in registers, and the polled form's rows of a warp (trsv_steps, trsv_block)
+  const bool dbl = sizeof(TV) == 8;
+  const int regs = dbl ? (plan.n_max <= 2 ? 2 : 4) : lpr == 2 ? (plan.n_max <= 16 ? 16 : 24) : plan.n_max <= 8 ? 8 : 16;
+  const int R = !dbl && lpr == 2 ? 2 : 4, lanes = 32 / R, per = 32 / lpr;
+  const FormCost C = form_cost(dbl, lpr, regs);
+  const double next = std::max(C.next, C.level / nwarps);  // fewer warps than steps under way
+  struct Group {  // a level of a slab
+    int32_t slab, steps, rows, longest, h0, h1, lev;
+  };
+  const int64_t ns = (int64_t)plan.hptr.size() - 1;
+  std::vector<Group> g;
+  std::vector<int32_t> of(P.npad, 0);  // group of every row
+  int64_t nlev = 0;
+  for (int64_t s = 0; s < ns; s++)
+    for (int32_t t = plan.step0[s], need = 0; t < plan.step0[s + 1];) {
+      const int32_t first = plan.head[t].first;
+      const int64_t r0 = s * rows + plan.row[(int64_t)t * per];
+      Group u{(int32_t)s, 0, 0, 0, plan.hptr[s] + need, 0, r0 < P.n ? P.lev[r0] : -1};
+      for (; t < plan.step0[s + 1] && plan.head[t].first == first; t++, u.steps++) {
+        const int nr = (int)(plan.head[t].shape & 63) / lpr;
+        for (int k = 0; k < nr; k++) of[s * rows + plan.row[(int64_t)t * per + k]] = (int32_t)g.size();
+        u.rows += nr;
+        u.longest = std::max(u.longest, (int32_t)(plan.head[t].shape >> 6 & 1023));
+        need = plan.head[t].need;
+      }
+      u.h1 = plan.hptr[s] + need;
+      if (u.lev < 0) continue;  // padding rows
+      nlev = std::max<int64_t>(nlev, u.lev + 1);
+      g.push_back(u);
+    }
+  std::vector<int32_t> at(nlev + 1, 0), order(g.size());
+  for (auto &u : g) at[lower ? u.lev + 1 : nlev - u.lev]++;
+  for (int64_t l = 0; l < nlev; l++) at[l + 1] += at[l];
+  for (size_t i = 0; i < g.size(); i++) order[at[lower ? g[i].lev : nlev - 1 - g[i].lev]++] = (int32_t)i;
+  std::vector<double> done(g.size()), pdone(g.size()), slab(ns, 0.0), pslab(ns, 0.0), copied(ns, 0.0);
+  Forecast f{0.0, 0.0};
+  for (int32_t i : order) {
+    const Group &u = g[i];
+    double b = slab[u.slab], pb = pslab[u.slab], c = copied[u.slab];
+    for (int32_t h = u.h0; h < u.h1; h++) {
+      const int32_t d = of[plan.hpos[h]];
+      c = std::max(c + C.halo, done[d]);
+      pb = std::max(pb, pdone[d] + C.phop);
+    }
+    if (u.h1 > u.h0) b = std::max(b, c + C.hop);
+    copied[u.slab] = c;
+    const int groups = (u.rows + R - 1) / R, entries = u.longest * lpr, passes = (groups + twarps - 1) / twarps;
+    const int over = std::max(0, (entries - TRSV_EPL * lanes + lanes - 1) / lanes);
+    slab[u.slab] = done[i] =
+        b + C.level + (u.steps - 1) * next + std::max(0, (u.longest + 3) / 4 - (regs + 3) / 4) * C.quad;
+    pslab[u.slab] = pdone[i] =
+        pb + C.plevel + (groups - 1) * C.pgroup + (passes - 1) * C.ppass + over * passes * C.poverflow;
+    f.steps = std::max(f.steps, done[i]);
+    f.polled = std::max(f.polled, pdone[i]);
+  }
+  return f;
+}
+
 #define NLE_STEPS(TV)                                                                              \
+  template Forecast forecast<TV>(const Permuted &, int64_t, bool, int, int, int, const StepsHost<TV> &); \
   template void plan_steps<TV>(const Permuted &, int64_t, bool, int, int, StepsHost<TV> &);       \
   template void build_steps<TV>(const Permuted &, int64_t, bool, int, StepsHost<TV> &);
 NLE_STEPS(float)

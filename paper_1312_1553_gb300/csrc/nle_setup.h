@@ -170,6 +170,25 @@ void plan_steps(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps
 template <typename TV>
 void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost<TV> &out);
 
+// Forecast of one solve in us, step form and polled form, for a plan with one
+// slab per solve slab: the steps of a plan, level by level, with the costs of
+// FormCost.  A level of a slab begins when the level before it is done and the values
+// it needs of other slabs are there.
+struct FormCost {
+  double level, next, hop, halo, quad;                // step form: first step of a level, each further one, a value on its
+                                                      // way to another slab, each halo value copied, each quad past the
+                                                      // registers
+  double plevel, pgroup, phop, ppass, poverflow;      // polled form: a level, each further group of rows, a value on its
+                                                      // way to another slab, a further pass of the warps over the level,
+                                                      // an overflow step
+};
+struct Forecast {
+  double steps, polled;
+};
+template <typename TV>
+Forecast forecast(const Permuted &P, int64_t rows, bool lower, int lpr, int nwarps, int twarps,
+                  const StepsHost<TV> &plan);
+
 // Chain schedule of the strictly lower (lower = true: P.Lrp/Lcol/Lval, levels
 // P.lev) or upper (P.Urp/Ucol/Uval, levels P.levU) factor for nwarps warps
 // per slab.  Needs the identity relabelling (slabs are ranges of the

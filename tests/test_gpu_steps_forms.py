@@ -50,6 +50,7 @@ def test_forms_give_the_same_bits(name, prec, rows):
         s = nle.Eigensolver(with_hub(A, neighbours), dict(precision=nle.NLE_MIXED if prec == "mixed" else nle.NLE_FP64,
                                                           trsv_schedule=nle.NLE_SCHED_LEVEL, trsv_rows=rows))
         s.factor_ic(lfil, tau)
+        assert (s.last_stats()["trsv_slabs"] > 0) == (neighbours == 3)
         out.append(np.stack([s.apply_prec(x).cpu().numpy()[:A.n] for x in g]))
         s.close()
     np.testing.assert_array_equal(out[0], out[1])
