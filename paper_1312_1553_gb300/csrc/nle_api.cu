@@ -566,6 +566,15 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
            both([&] { build_steps<TV>(P, h->bsize * h->steps, true, lpr, G[0]); },
                 [&] { build_steps<TV>(P, h->bsize * h->steps, false, lpr, G[1]); });
        });
+  // an earlier candidate may have been laid out in the other form: its buffers go
+  for (DBuf *b : {&h->L_off, &h->L_w, &h->L_col, &h->L_val, &h->L_round, &h->U_off, &h->U_w, &h->U_col, &h->U_val,
+                  &h->U_round})
+    if (h->steps) b->reset();
+  for (DBuf *b : {&h->L_wp, &h->L_task, &h->U_wp, &h->U_task})
+    if (!chain) b->reset();
+  for (auto &d : h->step_buf)
+    for (DBuf &b : d)
+      if (!h->steps) b.reset();
   if (with_a) {
     NLE_CUDA(h, upload(h->A_sptr, S.A.sptr, h->stream));
     NLE_CUDA(h, upload(h->A_col, S.A.col, h->stream));
