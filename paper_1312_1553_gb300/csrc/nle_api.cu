@@ -392,7 +392,10 @@ static Opts make_opts(nle_t h, double tol, int max_newton, int max_pcg) {
 static size_t slab_smem(nle_t h) {
   return (size_t)(h->steps ? h->bsize * h->steps + 1 + h->halo_n : 2 * h->bsize) * (mixed(h) ? 4 : 8);
 }
-constexpr size_t SLAB_SMEM_MAX = 192 * 1024;  // beside the kernels' static arrays (30 KB of 227)
+// The most of it, beside the kernels' static arrays (30 KB of 227).  Every launch
+// sets this limit, not its own size: the attribute belongs to the function, which handles
+// on other host threads launch too.
+constexpr size_t SLAB_SMEM_MAX = 192 * 1024;
 
 // The step form is taken where it is forecast (nle_setup.h) below this share of the
 // polled form's time.  A level costs it one hand-over where the polled form polls, but
@@ -444,7 +447,7 @@ static nle_status launch(nle_t h, int id, void **args) {
   void *fn = kernel_ptr<T>(id, h->rpc, h->chain);
   if (!fn) return fail(h, NLE_ERR_ARG, "no kernel instance for this size");
   const size_t dyn = slab_smem(h);
-  NLE_CUDA(h, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  NLE_CUDA(h, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SLAB_SMEM_MAX));
   int nb = 0;
   NLE_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, TPB, dyn));
   if (nb < 1 || h->grid > nb * h->nsm) return fail(h, NLE_ERR_CUDA, "persistent grid does not fit on the device");
@@ -964,7 +967,7 @@ nle_status nle_factor_ic(nle_t h, int lfil, double tau_ic) {
   // one slab of rows per CTA in the triangular solves (a multiple of TRSV_ROWS rows,
   // staged in shared memory)
   h->bsize = ((h->npad + TRSV_ROWS * grid - 1) / (TRSV_ROWS * grid)) * TRSV_ROWS;
-  if (2 * h->bsize * (int64_t)(mixed(h) ? 4 : 8) > 192 * 1024)
+  if (2 * h->bsize * (int64_t)(mixed(h) ? 4 : 8) > (int64_t)SLAB_SMEM_MAX)
     return fail(h, NLE_ERR_ARG, "n too large for the shared-memory slab of one persistent grid");
   const size_t tsz = mixed(h) ? 4 : 8;
   const int64_t ext = h->npad + 32 * h->vw;
@@ -1416,7 +1419,7 @@ static nle_status batch_impl(int count, nle_t *hs, int p, double tol, int max_ne
   Opts O = make_opts(h0, tol, max_newton, max_pcg);
   void *fn = kernel_ptr<T>(K_BATCH, rpc, h0->chain);
   if (!fn) return fail(h0, NLE_ERR_ARG, "no kernel instance for this size");
-  NLE_CUDA(h0, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  NLE_CUDA(h0, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SLAB_SMEM_MAX));
   int nb = 0;
   NLE_CUDA(h0, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, TPB, dyn));
   if (nb < 1) return fail(h0, NLE_ERR_CUDA, "batched kernel does not fit on an SM");
