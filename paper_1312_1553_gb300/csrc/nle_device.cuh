@@ -418,6 +418,87 @@ __device__ __forceinline__ void trsv_fetch(const TriEll<T> &M, int64_t b0, int64
   }
 }
 
+// --- pieces of the step form (trsv_steps) ---
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// shared-memory accesses by 32-bit address, kept in program order
+__device__ __forceinline__ void lds(unsigned a, float &v) {
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds(unsigned a, double &v) {
+  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ int4 lds4(unsigned a) {
+  int4 v;
+  asm volatile("ld.volatile.shared.v4.s32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts(unsigned a, float v) {
+  asm volatile("st.volatile.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, double v) {
+  asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void sts(unsigned a, int v) {
+  asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// Bound of a wait, asked every so many polls: true once spin_ns passed since
+// the first question or when another warp recorded an error.
+__device__ __forceinline__ bool wait_over(State *st, long long &t0, long long spin_ns, int where) {
+  const long long now = gtimer();
+  if (t0 == 0) t0 = now;
+  if (now - t0 > spin_ns) record_error(st, 8 /*NLE_ERR_TIMEOUT*/, where);
+  return ld_relaxed_int(&st->err) != 0;
+}
+
+// Copying warp m: its chunks of 32 halo values are m, m + COPY_WARPS, ...  One
+// chunk is in flight per warp: a pass over more of them costs every value
+// the whole pass, and the values arrive in nearly the order of the list.
+template <typename T>
+__device__ __forceinline__ void copy_halo(const int32_t *hpos, int nh, int m, const T *x, unsigned dst, Shared &sh,
+                                          long long spin_ns, State *st) {
+  const int lane = threadIdx.x & 31;
+  const unsigned flag = smem_addr(&sh.arrived[m]);
+  auto position = [&](int i) { return i < nh ? __ldg(hpos + i) : -1; };
+  int pos = position(32 * m + lane), ahead = position(32 * (m + COPY_WARPS) + lane);
+  bool over = false;  // a wait ran out: zeros for the rest, no further waits
+  for (int first = 32 * m; first < nh; first += 32 * COPY_WARPS) {
+    const unsigned to = dst + (unsigned)((first + lane) * (int)sizeof(T));
+    bool want = pos >= 0;
+    if (over && want) sts(to, T(0));
+    long long t0 = 0;
+    for (int it = 1; !over; it++) {
+      T v = T(0);
+      if (want) v = ld_relaxed(x + pos);
+      const bool got = want && !is_sent(v);
+      if (got) sts(to, v);
+      want = want && !got;
+      const unsigned left = __ballot_sync(0xffffffffu, want);
+      if (__any_sync(0xffffffffu, got)) {
+        __threadfence_block();
+        __syncwarp();
+        // all of this warp's values before the published one have arrived
+        if (lane == 0) sts(flag, left ? first + __ffs(left) - 1 : min(nh, first + 32 * COPY_WARPS));
+      }
+      if (!left) break;
+      if ((it & 4095) == 0 && __any_sync(0xffffffffu, wait_over(st, t0, spin_ns, 103))) {
+        if (want) sts(to, T(0));
+        over = true;
+      }
+    }
+    pos = ahead;
+    ahead = position(first + 64 * COPY_WARPS + lane);
+  }
+  __threadfence_block();
+  __syncwarp();
+  if (lane == 0) sts(flag, nh);
+}
+
 // Where a triangular solve reads its dependencies: its CTA's slab [b0, b1)
 // of the output x is copied in shared memory (stage); a dependency in
 // another slab is read from global memory.
