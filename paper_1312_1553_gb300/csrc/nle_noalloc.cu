@@ -42,17 +42,6 @@ constexpr int kRows = 4;    // rows a warp has open at a time, 32 / kRows lanes 
 constexpr int kLanes = 32 / kRows;
 constexpr int kSleep = 40;  // ns between two rounds of looks that found nothing
 
-// Quotient t / d given inv = 1 / d rounded: one corrected product where its
-// steps can neither overflow nor lose bits, the division otherwise.  Three
-// dependent FP64 instructions after t is known instead of the division's
-// dozen.
-__device__ __forceinline__ double quotient(double t, double d, double inv) {
-  const double q = t * inv;
-  const unsigned eq = ((unsigned)__double2hiint(q) >> 20) & 0x7ff, ed = ((unsigned)__double2hiint(d) >> 20) & 0x7ff;
-  if (eq - (1023u - 498u) > 996u || ed - (1023u - 332u) > 664u) return t / d;
-  return fma(fma(-q, d, t), inv, q);
-}
-
 // Four rows per warp, eight lanes a row and two entries of a lane in flight;
 // groups of four rows are taken round-robin in order (ascending for the lower
 // factor, descending for the upper one).  A row waits only for rows of earlier
@@ -135,7 +124,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_na_solve(int64_t n, const int32
         double s = acc;
 #pragma unroll
         for (int o = kLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-        if (publish && sub == 0) nle::st_relaxed(x + r, quotient(b - s, d, inv));
+        if (publish && sub == 0) nle::st_relaxed(x + r, nle::quotient(b - s, d, inv));
         if (publish) open = false;
         if (!__any_sync(kFull, open)) break;
         moved = true;

@@ -25,3 +25,25 @@ extern "C" int shim_wide(unsigned long long *bad) {
   cudaFree(d);
   return e == cudaSuccess ? 0 : 1;
 }
+
+__global__ void k_quotient(int n, const double *t, const double *d, double *q, double *div) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double inv = 1.0 / d[i];
+    q[i] = quotient(t[i], d[i], inv);
+    div[i] = t[i] / d[i];
+  }
+}
+
+// host arrays of n doubles
+extern "C" int shim_quotient(int n, const double *t, const double *d, double *q, double *div) {
+  double *dev = nullptr;
+  const size_t b = (size_t)n * sizeof(double);
+  if (cudaMalloc(&dev, 4 * b) != cudaSuccess) return 1;
+  cudaMemcpy(dev, t, b, cudaMemcpyHostToDevice), cudaMemcpy(dev + n, d, b, cudaMemcpyHostToDevice);
+  k_quotient<<<1216, 256>>>(n, dev, dev + n, dev + 2 * (size_t)n, dev + 3 * (size_t)n);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpy(q, dev + 2 * (size_t)n, b, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(div, dev + 3 * (size_t)n, b, cudaMemcpyDeviceToHost);
+  cudaFree(dev);
+  return e == cudaSuccess ? 0 : 1;
+}
