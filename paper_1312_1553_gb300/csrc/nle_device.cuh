@@ -501,13 +501,11 @@ __device__ __forceinline__ void copy_halo(const int32_t *hpos, int nh, int m, co
   const unsigned flag = smem_addr(&sh.arrived[m]);
   auto position = [&](int i) { return i < nh ? __ldg(hpos + i) : -1; };
   int pos = position(32 * m + lane), ahead = position(32 * (m + COPY_WARPS) + lane);
-  bool over = false;  // a wait ran out: zeros for the rest, no further waits
   for (int first = 32 * m; first < nh; first += 32 * COPY_WARPS) {
     const unsigned to = dst + (unsigned)((first + lane) * (int)sizeof(T));
     bool want = pos >= 0;
-    if (over && want) sts(to, T(0));
     long long t0 = 0;
-    for (int it = 1; !over; it++) {
+    for (int it = 1;; it++) {
       T v = T(0);
       if (want) v = ld_relaxed(x + pos);
       const bool got = want && !is_sent(v);
@@ -522,8 +520,11 @@ __device__ __forceinline__ void copy_halo(const int32_t *hpos, int nh, int m, co
       }
       if (!left) break;
       if ((it & 4095) == 0 && __any_sync(0xffffffffu, wait_over(st, t0, spin_ns, 103))) {
+        // zeros for the rest, and no further waits
         if (want) sts(to, T(0));
-        over = true;
+        for (first += 32 * COPY_WARPS; first < nh; first += 32 * COPY_WARPS)
+          if (first + lane < nh) sts(dst + (unsigned)((first + lane) * (int)sizeof(T)), T(0));
+        break;
       }
     }
     pos = ahead;
