@@ -400,22 +400,24 @@ constexpr size_t SLAB_SMEM_MAX = 192 * 1024;
 // The step form is taken where it is forecast (nle_setup.h) below this share of the
 // polled form's time.  A level costs it one hand-over where the polled form polls, but
 // its four copying warps bring in every value of another slab before it can be
-// used, 300 a microsecond, and the steps of a level follow one another: factors whose
-// slabs need several times their own rows from elsewhere (graphs in a random numbering)
-// and FP64 factors with wide levels are faster polled.  Measured, forecast ratio ->
-// one iteration of a whole solve, step form / polled form, us: FP64 60 x 70 0.66 -> 286 /
-// 422, 64^3 0.87 -> 1,064 / 1,315, 300 x 100 x 30 0.93 -> 1,328 / 1,486, 90^3 0.95 -> 1,825 / 1,934, graph of
-// 9,000 nodes 0.98 -> 214 / 201, 100^3 1.00 -> 2,291 / 2,226, graph of 20,000 1.25 -> 275 / 216; mixed
-// 100^3 0.59 -> 1,083 / 1,786, graph of 9,000 0.77 -> 181 / 203, of 20,000 1.16 -> 302 / 252, of
-// 35,000 1.46 -> 383 / 258.
+// used, 300 to 500 a microsecond, and the steps of a level follow one another: factors
+// whose slabs need several times their own rows from elsewhere (graphs in a random
+// numbering) and FP64 factors with wide levels are faster polled.  Measured, forecast ratio
+// -> one iteration of a whole solve, step form / polled form, us: mixed 100^3 0.59 -> 1,083 /
+// 1,786, graph of 9,000 nodes 0.77 -> 181 / 203, of 20,000 1.16 -> 302 / 252, of 35,000 1.46 -> 383 /
+// 258; FP64 60 x 70 0.63 -> 286 / 422, 64^3 0.83 -> 1,064 / 1,315, 300 x 100 x 30 0.89 -> 1,328 / 1,486,
+// 90^3 0.90 -> 1,825 / 1,934, 100^3 0.94 -> 2,291 / 2,226, graph of 9,000 1.04 -> 214 / 201.
+// Graphs of 6,000 and 30,000 nodes on 4 and 8 CTAs, FP64, 0.88 -> 213 / 225 (in a batch 287 /
+// 280) and 0.94 -> 647 / 567.
 // The levels of a multicolour ordering go back and forth between the slabs, which
-// the forecast takes too lightly, in FP64 above all: 600 x 700, distance 1 0.67 -> 2,232 /
-// 2,838, 32^3 0.75 -> 486 / 580, 64^3 0.83 -> 1,257 / 1,203, 100^3 0.91 -> 2,468 / 2,278, 600 x 700,
-// distance 2 1.06 -> 2,121 / 1,740; mixed 27-point 48^3 0.87 -> 1,948 / 2,469, 32^3 0.88 -> 403 / 363,
-// 100^3 0.96 -> 2,510 / 1,797.
+// the forecast takes too lightly: FP64 600 x 700, distance 1 0.69 -> 2,232 / 2,838, 32^3 0.76 ->
+// 486 / 580, 45^3 0.89 -> 741 / 708, 64^3 0.92 -> 1,257 / 1,203, 600 x 700, distance 2 0.99 -> 2,121 /
+// 1,740; mixed 27-point 48^3 0.87 -> 1,948 / 2,469, 32^3 0.88 -> 403 / 363, 100^3 0.96 -> 2,510 / 1,797.
 // Merged slabs (m > 1 below) have narrow levels and are not asked: 0.46 to 0.98 of
 // the polled time on the same matrices.
-static double step_gain(bool multicolor, bool fp64) { return !multicolor ? 0.965 : fp64 ? 0.78 : 0.875; }
+static double step_gain(nle_t h, bool multicolor) {
+  return mixed(h) ? (multicolor ? 0.875 : 0.965) : multicolor ? 0.85 : 0.92;
+}
 
 // Slabs per solve slab: a value takes about 1 us from one solve slab to the
 // next, so fewer of them are better as long as a level still is one step of
@@ -553,7 +555,8 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
       };
       both([&] { plan(0); }, [&] { plan(1); });
       if (!G[0].fits || !G[1].fits) break;
-      if (fc[0].steps + fc[1].steps > step_gain(level_rounds, sizeof(TV) == 8) * (fc[0].polled + fc[1].polled)) break;
+      const double gain = step_gain(h, level_rounds);
+      if (fc[0].steps + fc[1].steps > gain * (fc[0].polled + fc[1].polled)) break;
       for (int d = 0; d < 2; d++) {
         h->halo_n = (int)std::max<int64_t>(h->halo_n, G[d].halo_max);
         h->step_n = std::max(h->step_n, G[d].n_max);

@@ -567,13 +567,13 @@ void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost
 }
 
 // Costs in us, fitted to one application of (L L^T)^{-1} on 7-point (20^3 to
-// 106^3), 5-point, 27-point and random geometric graph factors, natural and both
-// multicolour orderings: the forecasts of 67 measured times each miss by 8 to
-// 15 % (root mean square).
+// 106^3), 5-point, 27-point and random geometric graph factors (4, 8 and all
+// CTAs), natural and both multicolour orderings: the forecasts of 83 measured times
+// each miss by 8 to 14 % (root mean square).
 static FormCost form_cost(bool dbl, int lpr, int regs) {
-  if (dbl) return {regs <= 2 ? 0.36 : 0.41, 0.065, 0.80, 0.0030, 0.36, 0.63, 0.004, 0.38, 0.85, 0.47};
-  if (lpr == 2) return {0.16, 0.084, 0.65, 0.0033, 0.19, 0.29, 0.018, 0.71, 0.39, 0.29};
-  return {regs <= 8 ? 0.086 : 0.146, 0.12, 0.65, 0.0034, 0.20, 0.29, 0.022, 0.63, 0.25, 0.40};
+  if (dbl) return {regs <= 2 ? 0.34 : 0.40, 0.064, 0.66, 0.0021, 0.40, 0.21, 0.63, 0.007, 0.31, 0.85, 0.48};
+  if (lpr == 2) return {0.16, 0.084, 0.65, 0.0033, 0.19, 0.0, 0.29, 0.018, 0.71, 0.39, 0.29};
+  return {regs <= 8 ? 0.086 : 0.146, 0.12, 0.65, 0.0034, 0.20, 0.0, 0.29, 0.022, 0.63, 0.25, 0.40};
 }
 
 template <typename TV>
@@ -627,8 +627,8 @@ Forecast forecast(const Permuted &P, int64_t rows, bool lower, int lpr, int nwar
     copied[u.slab] = c;
     const int groups = (u.rows + R - 1) / R, entries = u.longest * lpr, passes = (groups + twarps - 1) / twarps;
     const int over = std::max(0, (entries - TRSV_EPL * lanes + lanes - 1) / lanes);
-    slab[u.slab] = done[i] =
-        b + C.level + (u.steps - 1) * next + std::max(0, (u.longest + 3) / 4 - (regs + 3) / 4) * C.quad;
+    const int quads = std::max(0, (u.longest + 3) / 4 - (regs + 3) / 4);
+    slab[u.slab] = done[i] = b + C.level + quads * C.quad + (u.steps - 1) * (next + quads * C.nquad);
     pslab[u.slab] = pdone[i] =
         pb + C.plevel + (groups - 1) * C.pgroup + (passes - 1) * C.ppass + over * passes * C.poverflow;
     f.steps = std::max(f.steps, done[i]);

@@ -175,12 +175,12 @@ void build_steps(const Permuted &P, int64_t rows, bool lower, int lpr, StepsHost
 // FormCost.  A level of a slab begins when the level before it is done and the values
 // it needs of other slabs are there.
 struct FormCost {
-  double level, next, hop, halo, quad;                // step form: first step of a level, each further one, a value on its
-                                                      // way to another slab, each halo value copied, each quad past the
-                                                      // registers
-  double plevel, pgroup, phop, ppass, poverflow;      // polled form: a level, each further group of rows, a value on its
-                                                      // way to another slab, a further pass of the warps over the level,
-                                                      // an overflow step
+  double level, next, hop, halo, quad, nquad;     // step form: first step of a level, each further one, a value on its
+                                                  // way to another slab, each halo value copied, each quad past the
+                                                  // registers in the first step and in each further one
+  double plevel, pgroup, phop, ppass, poverflow;  // polled form: a level, each further group of rows, a value on its
+                                                  // way to another slab, a further pass of the warps over the level,
+                                                  // an overflow step
 };
 struct Forecast {
   double steps, polled;
