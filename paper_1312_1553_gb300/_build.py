@@ -1,8 +1,8 @@
 """Build of the nle CUDA library (libnle.so) for sm_103a.
 
-The kernels are compiled once per (precision, rows-per-thread, triangular-
-solve schedule) triple in parallel translation units, then linked with the C ABI and the host set-up
-code into ``paper_1312_1553_gb300/libnle.so``.  Objects go to ``_build/`` at
+The kernels are compiled once per (precision, rows-per-thread, triangular
+solves) triple in parallel translation units, then linked with the C ABI and the
+host set-up code into ``paper_1312_1553_gb300/libnle.so``.  Objects go to ``_build/`` at
 the repository root.  A stamp over the sources and flags skips rebuilds.
 """
 from __future__ import annotations
@@ -22,9 +22,10 @@ LIB = os.path.join(HERE, "libnle.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
            "--expt-relaxed-constexpr"] + ARCH
-# (tag, precision, rows-per-thread chunks, chain schedule of the triangular solves)
-VARIANTS = [(f"{p}{r}{'c' if c else ''}", t, r, c) for c in (0, 1) for p, t in (("f", "float"), ("d", "double"))
-            for r in (1, 2, 4, 8)]
+# (tag, precision, rows-per-thread chunks, triangular solves: 0 level schedule with
+# both forms, 1 chain schedule, 2 level schedule without the step form)
+VARIANTS = [(f"{p}{r}{'cp'[c - 1:c]}", t, r, c) for c in (0, 2, 1) for r in (8, 4, 2, 1)
+            for p, t in (("d", "double"), ("f", "float"))]
 
 
 def _nvcc() -> str:
@@ -61,10 +62,10 @@ def build(force: bool = False, jobs: int | None = None, verbose: bool = False) -
     cmds = []
     objs = []
     kern = os.path.join(CSRC, "nle_kernels.cu")
-    for tag, typ, rpc, chain in VARIANTS:
+    for tag, typ, rpc, trsv in VARIANTS:
         o = os.path.join(BUILD, f"nle_kernels_{tag}.o")
         cmds.append([nvcc, *NVFLAGS, f"-DNLE_T={typ}", f"-DNLE_RPC={rpc}", f"-DNLE_TAG={tag}",
-                     f"-DNLE_CHAIN_TU={chain}", "-c", kern, "-o", o])
+                     f"-DNLE_TRSV_TU={trsv}", "-c", kern, "-o", o])
         objs.append(o)
     for src in ("nle_api.cu", "nle_setup.cpp", "nle_noalloc.cu", "nle_ict.cu"):
         o = os.path.join(BUILD, src.replace(".", "_") + ".o")

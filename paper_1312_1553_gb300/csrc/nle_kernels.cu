@@ -220,15 +220,15 @@ __device__ bool gram(const Dev<T> &D, Shared &sh, Ctl &ctl, int m, int k) {
 // ---------------------------------------------------------------------------
 extern __shared__ __align__(16) unsigned char nle_dyn_smem[];  // two slabs of the triangular solves
 
-// Schedule of the triangular solves compiled into this translation unit
-// (the build compiles every (precision, rows-per-thread) pair once per
-// schedule, so each kernel holds one solve only and keeps its registers);
-// the kernels carry it as a template argument so that the two builds'
-// kernels have distinct names.
-#ifndef NLE_CHAIN_TU
-#define NLE_CHAIN_TU 0
+// Triangular solves compiled into this translation unit: 0 the level schedule
+// with both forms, 1 the chain schedule, 2 the level schedule's polled form alone
+// (the build compiles every (precision, rows-per-thread) pair once for each, so
+// that the chain and the polled solves keep their registers); the kernels carry
+// it as a template argument so that the builds' kernels have distinct names.
+#ifndef NLE_TRSV_TU
+#define NLE_TRSV_TU 0
 #endif
-constexpr bool kChainTU = NLE_CHAIN_TU != 0;
+constexpr bool kChainTU = NLE_TRSV_TU == 1, kStepTU = NLE_TRSV_TU == 0;
 
 // ---------------------------------------------------------------------------
 // Step form of the level schedule, one solve slab of rows per CTA.
@@ -578,7 +578,7 @@ __device__ __forceinline__ void steps_solve(const Dev<T> &D, Shared &sh, const C
 
 template <typename T>
 __device__ __forceinline__ bool trsv_forward(const Dev<T> &D, Shared &sh, Ctl &ctl, int k) {
-  if constexpr (!kChainTU) {
+  if constexpr (kStepTU) {
     if (D.steps) {
       if (k == 0) {
         steps_solve<true, T>(D, sh, ctl, D.g);
@@ -632,7 +632,7 @@ __device__ __forceinline__ bool trsv_forward(const Dev<T> &D, Shared &sh, Ctl &c
 // solves.
 template <typename T>
 __device__ __forceinline__ void trsv_backward(const Dev<T> &D, Shared &sh, const Ctl &ctl) {
-  if constexpr (!kChainTU) {
+  if constexpr (kStepTU) {
     if (D.steps) {
       steps_solve<false, T>(D, sh, ctl, D.z);
       return;
@@ -1863,8 +1863,8 @@ __global__ void __launch_bounds__(TPB, 1) k_batch(Batch<T> B, Opts O) {
 }
 
 // ---------------------------------------------------------------------------
-// host-side launch table.  This file is compiled once per (precision, RPC)
-// pair (NLE_T, NLE_RPC, NLE_TAG defined by the build) so that the
+// host-side launch table.  This file is compiled once per (precision, RPC,
+// triangular solves) triple (NLE_T, NLE_RPC, NLE_TRSV_TU, NLE_TAG defined by the build) so that the
 // instantiations compile in parallel.
 // ---------------------------------------------------------------------------
 #if defined(NLE_T) && defined(NLE_RPC) && defined(NLE_TAG)
@@ -1872,13 +1872,13 @@ __global__ void __launch_bounds__(TPB, 1) k_batch(Batch<T> B, Opts O) {
 #define NLE_CAT(a, b) NLE_CAT2(a, b)
 void *NLE_CAT(kernel_ptr_, NLE_TAG)(int id) {
   switch (id) {
-    case 0: return (void *)k_newton<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
-    case 1: return (void *)k_dacg<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
-    case 2: return (void *)k_shifted<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
-    case 3: return (void *)k_prec<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
-    case 4: return (void *)k_pcg<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
-    case 5: return (void *)k_adjoint<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
-    case 6: return (void *)k_batch<NLE_T, NLE_RPC, NLE_CHAIN_TU>;
+    case 0: return (void *)k_newton<NLE_T, NLE_RPC, NLE_TRSV_TU>;
+    case 1: return (void *)k_dacg<NLE_T, NLE_RPC, NLE_TRSV_TU>;
+    case 2: return (void *)k_shifted<NLE_T, NLE_RPC, NLE_TRSV_TU>;
+    case 3: return (void *)k_prec<NLE_T, NLE_RPC, NLE_TRSV_TU>;
+    case 4: return (void *)k_pcg<NLE_T, NLE_RPC, NLE_TRSV_TU>;
+    case 5: return (void *)k_adjoint<NLE_T, NLE_RPC, NLE_TRSV_TU>;
+    case 6: return (void *)k_batch<NLE_T, NLE_RPC, NLE_TRSV_TU>;
   }
   return nullptr;
 }
