@@ -677,7 +677,8 @@ __device__ __noinline__ void trsv_block_r(const TriEll<T> &M, T *x, int64_t npad
 // (4, or 2 for factors with wide rows), each a compile-time instance.  The
 // instances are called, not inlined: inside the persistent solver kernels
 // the inlined solves raised register spills and measured 4-10 % slower per
-// whole solve (the call happens once per triangular solve).
+// whole solve (the call happens once per triangular solve; the step form is
+// the other way round, see trsv_steps).
 template <bool LOWER, typename T, typename RHS>
 __device__ __forceinline__ void trsv_block(const TriEll<T> &M, T *x, int64_t npad, int64_t bsize, int twarps,
                                            long long spin_ns, int poll_ns, State *st, T *stage_mem, RHS rhs_of) {
