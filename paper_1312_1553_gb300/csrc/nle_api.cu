@@ -541,7 +541,7 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
         if (m == 1 && G[d].fits)
           fc[d] = forecast<TV>(P, h->bsize, d == 0, lpr, h->step_warps, h->opt.trsv_warps, G[d]);
       };
-      both([&] { plan(0); }, [&] { plan(1); });
+      both(P.n, [&] { plan(0); }, [&] { plan(1); });
       if (!G[0].fits || !G[1].fits) break;
       const double gain = step_gain(h, level_rounds);
       if (fc[0].steps + fc[1].steps > gain * (fc[0].polled + fc[1].polled)) break;
@@ -554,10 +554,10 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
       h->steps = 0;
     }
   }
-  both([&] { build_sell<TV>(P, H, h->bsize, level_rounds, h->trows, S, !h->steps && !chain, with_a); },
+  both(P.n, [&] { build_sell<TV>(P, H, h->bsize, level_rounds, h->trows, S, !h->steps && !chain, with_a); },
        [&] {
          if (h->steps)
-           both([&] { build_steps<TV>(P, h->bsize * h->steps, true, lpr, G[0]); },
+           both(P.n, [&] { build_steps<TV>(P, h->bsize * h->steps, true, lpr, G[0]); },
                 [&] { build_steps<TV>(P, h->bsize * h->steps, false, lpr, G[1]); });
        });
   // an earlier candidate may have been laid out in the other form: its buffers go
@@ -579,7 +579,8 @@ static nle_status upload_layout(nle_t h, const Permuted &P, bool level_rounds, i
   if (chain) {
     const int nw = std::max(1, std::min(NWARP, h->opt.trsv_warps));
     ChainHost<TV> CL, CU;
-    both([&] { build_chain<TV>(P, h->bsize, true, nw, CL); }, [&] { build_chain<TV>(P, h->bsize, false, nw, CU); });
+    both(P.n, [&] { build_chain<TV>(P, h->bsize, true, nw, CL); },
+         [&] { build_chain<TV>(P, h->bsize, false, nw, CU); });
     h->nstrands = CL.nstrands;
     S.L = std::move(CL.ell);
     S.U = std::move(CU.ell);

@@ -882,7 +882,7 @@ void permute(int64_t n, const int64_t *rp, const int32_t *ci, const double *va, 
       P.Urp[i + 1] = (int64_t)P.Ucol.size();
     }
   };
-  both(matrix, [&] { both(lower, upper); });
+  both(n, matrix, [&] { both(n, lower, upper); });
 }
 
 }  // namespace nle

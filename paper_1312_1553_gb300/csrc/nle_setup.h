@@ -146,15 +146,23 @@ template <typename TV>
 void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int R, SellSet<TV> &S,
                 bool with_ell = true, bool with_a = true);
 
-// Run a and b, a on a thread of its own where one can be had.  An exception of
-// either leaves only after both have ended.
+// Run a and b, set-up work on n rows, a on a thread of its own where that pays
+// and one can be had.  An exception of either leaves only after both have ended.
+// Below THREAD_ROWS a thread costs more than it saves: set-up of 100 rows, fixed
+// schedule, 0.72 ms without threads, 0.88 with, of 1,110 rows 2.28 and 2.37; 27,000 rows 13.6
+// and 12.7.
+constexpr int64_t THREAD_ROWS = 4096;
 template <typename FA, typename FB>
-void both(FA a, FB b) {
+void both(int64_t n, FA a, FB b) {
   std::future<void> f;
-  try {
-    f = std::async(std::launch::async, [&a] { a(); });
-  } catch (const std::system_error &) {
+  if (n < THREAD_ROWS) {
     a();
+  } else {
+    try {
+      f = std::async(std::launch::async, [&a] { a(); });
+    } catch (const std::system_error &) {
+      a();
+    }
   }
   b();
   if (f.valid()) f.get();
