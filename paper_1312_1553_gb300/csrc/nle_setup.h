@@ -149,8 +149,8 @@ void build_sell(const Permuted &P, int H, int64_t bsize, bool level_rounds, int 
 // Run a and b, set-up work on n rows, a on a thread of its own where that pays
 // and one can be had.  An exception of either leaves only after both have ended.
 // Below THREAD_ROWS a thread costs more than it saves: set-up of 100 rows, fixed
-// schedule, 0.72 ms without threads, 0.88 with, of 1,110 rows 2.28 and 2.37; 27,000 rows 13.6
-// and 12.7.
+// schedule, 0.72 ms without threads, 0.88 with, of 1,110 rows 2.29 and 2.37; at 4,200 rows the
+// set-up with threads takes what it took before there were any (4.8 ms).
 constexpr int64_t THREAD_ROWS = 4096;
 template <typename FA, typename FB>
 void both(int64_t n, FA a, FB b) {
